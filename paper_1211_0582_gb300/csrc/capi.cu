@@ -204,11 +204,12 @@ int dg_mesh_upload(dg_ctx *ctx, int64_t Nv, const double *VX, const double *VY, 
   cudaStream_t s = ctx->stream;
 
   // host-side operator layouts for the CUDA-core kernels
-  std::vector<float> DT(size_t(3) * Np * Npad, 0.f), LT(size_t(4) * Nfp * Npad, 0.f);
+  // (rows read ahead of their use and past a row's end: three rows of padding)
+  std::vector<float> DT(size_t(3) * (Npad + 1) * Npad, 0.f), LT(size_t(4 * Nfp + 3) * Npad, 0.f);
   const std::vector<double> *Ds[3] = {&o.Dr, &o.Ds, &o.Dt};
   for (int d = 0; d < 3; ++d)
     for (int j = 0; j < Np; ++j)
-      for (int i = 0; i < Np; ++i) DT[(size_t(d) * Np + j) * Npad + i] = float((*Ds[d])[i * Np + j]);
+      for (int i = 0; i < Np; ++i) DT[(size_t(3) * j + d) * Npad + i] = float((*Ds[d])[i * Np + j]);
   for (int m = 0; m < 4 * Nfp; ++m)
     for (int i = 0; i < Np; ++i) LT[size_t(m) * Npad + i] = float(o.LIFT[i * 4 * Nfp + m]);
   std::vector<uint8_t> tab(4 * Nfp + 2 * kConnKinds * Nfp);

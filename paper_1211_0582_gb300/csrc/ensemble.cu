@@ -114,7 +114,8 @@ std::string cache_path() {
 
 std::string cache_key(const EnsembleState &st, int N, int precision, int64_t K) {
   std::ostringstream os;
-  os << st.gpu << "|N=" << N << "|P=" << precision << "|K=" << K;
+  // T: the candidate list that the cached index refers to
+  os << st.gpu << "|N=" << N << "|P=" << precision << "|K=" << K << "|T=2";
   return os.str();
 }
 

@@ -1,272 +1,455 @@
 // FP32 CUDA-core form of the fused right-hand side / LSERK stage.
 //
-// One block owns EB consecutive elements and runs the paper's four subtasks
-// (Section 2, Fig. dg-subtasks) on them without leaving the SM:
-//   1. stage the block's fields u[6][EB][Npad] in shared memory (float4 loads,
-//      coalesced because each field's element rows are contiguous);
-//   2. local differentiation: thread (element e, node quad q) forms
-//      u_r, u_s, u_t = D_{r,s,t} u for its four nodes and six fields, then the
-//      chain rule (eq. dg-reference-matrices) and the curls;
-//   3. flux gather (eq. num-flux): interior trace from shared memory,
-//      exterior trace from the neighbour's row (L2), PEC mirror on walls,
-//      upwind flux with the face's precomputed impedance weights (Fscale
-//      included), into shared memory;
-//   4. flux lifting: LIFT (Np x 4Nfp) times the face fluxes, added to the
-//      curls and scaled by 1/eps, 1/mu;
-// then either stores the right-hand side or applies the low-storage RK
-// update res = a res + dt rhs, u_out = u + b res (operator assembly).
-// The transposed operators D^T[j][i], LIFT^T[m][i] are read as float4 along i
-// through the read-only cache; they are small and stay cache resident. The
-// launch is persistent (blocks loop over element tiles) with the elements per
-// block picked per order from measurements: 128 / (Np_pad / 4), 80 / (...) at
-// N = 4.
+// One block owns a tile of EB consecutive elements and runs the paper's four
+// subtasks (Section 2, Fig. dg-subtasks) on it without leaving the SM, as ONE
+// matrix product over the tile's (element, field) rows:
+//   out[(e,c), i] = sum_k X[k, (e,c)] W[k, i],   W = [LIFT^T; D^T],
+// where the curl is taken before the differentiation: for node j and direction
+// d the row (e, c) of X holds the two-field combination sum_l +-(dr_d/dx_l) u_l
+// whose derivative along d belongs to component c of curl H or -curl E (eq.
+// dg-reference-matrices; the metric terms are constant per element), and for
+// the lifting it holds the face node's flux. All products go into the same
+// accumulators (24 per element and node quad, where three derivatives of six
+// fields take 72), so a thread can hold two elements x two node quads and
+// reads 12 X and 8 W values per 96 multiply-adds.
+//
+// X is built chunk by chunk in shared memory, [k][row] with rows e * 6 + c: the
+// fluxes of FR face nodes, then QC node quads times three directions. W is
+// staged beside it by asynchronous copies from L2 that run while X is built:
+// read through L1 instead, a 16-byte load that several lanes share costs up to
+// 8 data-pipe cycles (from shared memory two), and the operators crowd the
+// neighbours' traces out of L1.
+//
+// What bounds it: at N >= 4 the FP32 pipe (53-57% of its cycles busy; packed
+// FMAs with operands from shared memory reach 80-85% in isolation) and the
+// latencies of the traces and of the update that the blocks of an SM do not
+// cover for each other; at N <= 3 those latencies. Measured (us per stage
+// before, with three derivatives per field and the operators read through L1,
+// and now): N=1 162,000 tets 48.8 -> 33.4; N=2 131,712 tets 119 -> 73; N=3
+// 131,712 tets 203 -> 146; N=4 82,944 tets 298 -> 204; N=5 82,944 tets 479 ->
+// 394; N=6 24,576 tets 292 -> 227; N=7 24,576 tets 522 -> 422; N=8 24,576 tets
+// 859 -> 684; N=9 10,368 tets 668 -> 507; 162 tets at N=3 14.8 -> 6.6, 1,296
+// tets at N=5 21.1 -> 17.
 #pragma once
 #include <atomic>
+#include <cmath>
 
 #include "common.cuh"
 #include "flux.cuh"
+#include "tiles.cuh"
 
 namespace dgmx {
 
-// Elements per block of the single-mesh launch (measured best on GB300).
-template <int N>
-constexpr int simt_default_eb() {
-  return (N == 4 ? 80 : 128) / Dims<N>::NQ > 0 ? (N == 4 ? 80 : 128) / Dims<N>::NQ : 1;
-}
-
-template <int N, int EB_ = simt_default_eb<N>()>
-struct SimtCfg {
+// Shape of a launch: elements per tile and products per thread, RE elements x
+// CQ node quads (6 RE x 4 CQ accumulators).
+//   SMALL: one element x one quad and few, long chunks. A thread's chain of
+//     products and a tile's chain of barriers are short, which is what counts
+//     while a launch has only a few tiles per SM; at N <= 3 and N = 6 it is
+//     the faster one at every size.
+//   otherwise two elements x two quads: half the shared-memory reads per
+//     product, but a tile takes as long with one element as with all of them.
+template <int N, bool SMALL>
+struct SimtShape {
   using D = Dims<N>;
-  static constexpr int EB = EB_;                         // elements per block
-  static constexpr int NT = (EB * D::NQ + 31) / 32 * 32; // threads per block
-  static constexpr size_t SMEM =
-      (size_t(6) * EB * D::NPP + size_t(6) * EB * D::NFF) * 4 + ((100 * D::NFP + 15) / 16) * 16;
+  static constexpr int RE = SMALL ? 1 : 2, CQ = SMALL ? 1 : 2;
+  static constexpr int CG = (D::NQ + CQ - 1) / CQ; // column groups: node quads cg and (CQ = 2) cg + CG
+  // element groups of a block (even: neighbouring lanes hold two of them)
+  static constexpr int GROUPS = SMALL ? (N == 1 ? 64 : N <= 3 ? 32 : N == 4 ? 16 : N == 5 || N == 7 ? 8 : N == 6 ? 12
+                                         : N == 8 ? 6 : 4)
+                                      : 128 / CG / 2 * 2;
+  static constexpr int EB = RE * GROUPS;
+  // Rows of X per chunk: FR face nodes (even, as 4 Nfp is) or QC node quads
+  // (12 rows each).
+  static constexpr int FR = SMALL ? (N == 9 ? 44 : N == 8 ? 60 : N == 7 ? 72 : D::NFF)
+                                  : N == 9 ? 44 : N == 8 ? 60 : N == 7 ? 72 : N == 5 ? 42 : 30;
+  static constexpr int QC = SMALL ? (N == 9 ? 5 : N == 8 ? 7 : N == 7 ? 6 : N == 6 || N == 5 ? 7 : D::NQ)
+                                  : N == 9 ? 4 : N == 8 ? 5 : N == 7 ? 6 : N == 5 ? 4 : 2;
 };
 
-// Field loads: from L2, bypassing L1 (fields are streamed once and the
-// neighbour traces hit L2 anyway; L1 stays with the operator matrices), or
-// through the read-only path (measured slower). Persistent multi-stage kernels
-// need the L2 path for coherence: other blocks wrote the data in an earlier stage.
-template <bool COHERENT>
-__device__ __forceinline__ float4 load_field4(const float *p) {
-  if constexpr (COHERENT) return __ldcg(reinterpret_cast<const float4 *>(p));
-  else return ldg4(p);
+// Orders that only the small shape serves.
+template <int N>
+constexpr bool simt_small_only() {
+  return N <= 3 || N == 6;
 }
+
+template <int N, bool SMALL, int EB_ = SimtShape<N, SMALL>::EB>
+struct SimtCfg {
+  using D = Dims<N>;
+  using S = SimtShape<N, SMALL>;
+  static constexpr int EB = EB_;
+  static_assert(EB % (2 * S::RE) == 0 && EB <= S::EB, "whole pairs of element groups");
+  static constexpr int QC = S::QC, FR = S::FR, CG = S::CG;
+  static constexpr int NT = EB / S::RE * CG > 128 ? (EB / S::RE * CG + 31) / 32 * 32 : 128; // threads per block
+  // Row stride of X: an odd multiple of 4 floats (16-byte loads along the rows
+  // are aligned, the stores of neighbouring nodes fall into different banks)
+  static constexpr int RS = (6 * EB) % 8 == 4 ? 6 * EB : 6 * EB + 4;
+  static constexpr int WS = D::NPP;                      // row stride of the staged operator
+  static constexpr int XR = 12 * QC > FR ? 12 * QC : FR; // rows of X
+  // bytes: X and the operator rows of the chunk, face data of the tile, metric
+  // terms, reference values, node tables
+  static constexpr int OFF_W = XR * RS * 4;
+  static constexpr int OFF_FGEO = OFF_W + XR * WS * 4; // float4 [EB * 4]
+  static constexpr int OFF_FMAT = OFF_FGEO + EB * 64;  // float4 [EB * 4]
+  static constexpr int OFF_FCONN = OFF_FMAT + EB * 64; // int2 [EB * 4]
+  static constexpr int OFF_G = OFF_FCONN + EB * 32;    // float [EB][GS]
+  static constexpr int GS = 12;                        // row stride of the metric terms
+  static constexpr int OFF_REF = OFF_G + EB * GS * 4;  // float [EB][6]
+  static constexpr int OFF_TAB = OFF_REF + EB * 24;
+  static constexpr size_t SMEM = size_t(OFF_TAB + (100 * D::NFP + 15) / 16 * 16);
+  // blocks per SM asked for: three of 168 registers per thread, or (SMALL) as
+  // many of 128 as shared memory holds
+  static constexpr int FIT = int(228 * 1024 / (SMEM + 1024)) < 512 / NT ? int(228 * 1024 / (SMEM + 1024)) : 512 / NT > 0 ? 512 / NT : 1;
+  static constexpr int MINB = SMALL ? FIT : 3;
+  static_assert(SMEM <= 228 * 1024 / MINB - 1024, "MINB blocks per SM");
+};
+
+// Field loads. Tile rows come from L2 past L1 (used once or twice); the face
+// nodes' scattered reads hit the same lines again and go through L1. A
+// persistent multi-stage launch (COHERENT) reads everything from L2: other
+// blocks wrote the data in an earlier stage.
+__device__ __forceinline__ float4 load_field4(const float *p) { return __ldcg(reinterpret_cast<const float4 *>(p)); }
 template <bool COHERENT>
-__device__ __forceinline__ float load_field(const float *p) {
+__device__ __forceinline__ float load_trace(const float *p) {
   if constexpr (COHERENT) return __ldcg(p);
   else return __ldg(p);
 }
 
-// One block-tile of EB elements starting at k0 (all threads of the block call it).
-template <int N, int MODE, int EB, bool COHERENT>
-__device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, float4 *smem4) {
-  using D = Dims<N>;
-  using Cfg = SimtCfg<N, EB>;
-  constexpr int NP = D::NP, NFP = D::NFP, NPP = D::NPP, NQ = D::NQ, NFF = D::NFF;
-  constexpr int NT = Cfg::NT;
-  float *s_u = reinterpret_cast<float *>(smem4);             // [6][EB][NPP]
-  float *s_fl = s_u + 6 * EB * NPP;                          // [6][EB][NFF]
-  uint8_t *s_fm = reinterpret_cast<uint8_t *>(s_fl + 6 * EB * NFF); // [NFF]
-  uint8_t *s_nb = s_fm + NFF;                                // [96][NFP]
+// The node tables of a block (once per launch; the first tile's barrier orders them).
+template <class Cfg>
+__device__ __forceinline__ void simt_setup(const StageArgs &a, float4 *smem4) {
+  using D = typename Cfg::D;
+  uint8_t *tab = reinterpret_cast<uint8_t *>(smem4) + Cfg::OFF_TAB;
+  for (int i = threadIdx.x; i < D::NFF + kConnKinds * D::NFP; i += Cfg::NT)
+    tab[i] = i < D::NFF ? a.fmask[i] : a.nbrtab[i - D::NFF];
+}
 
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void *dst, const void *src) {
+  if constexpr (BYTES == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(uint32_t(__cvta_generic_to_shared(dst))), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(uint32_t(__cvta_generic_to_shared(dst))), "l"(src), "n"(BYTES) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// kc contiguous operator rows into shared memory, asynchronously.
+template <class Cfg>
+__device__ __forceinline__ void simt_stage_operator(float *s_w, const float *__restrict__ w, int kc) {
+  for (int i = threadIdx.x; i < kc * Cfg::D::NQ; i += Cfg::NT) cp_async<16>(s_w + 4 * i, w + 4 * i);
+}
+
+// acc[p][n] += (X[k][2p], X[k][2p+1]) W[k][n] over kc rows k (kc even): packed
+// FP32 pairs along the rows, the operator value broadcast to both halves. The
+// operands of the next row are requested before the current row's products.
+template <class Cfg>
+__device__ __forceinline__ void simt_product(float2 (&acc)[3 * Cfg::S::RE][4 * Cfg::S::CQ], const float *x,
+                                             const float *w, int kc) {
+  constexpr int RE = Cfg::S::RE, CQ = Cfg::S::CQ;
+  float2 x0[3 * RE], x1[3 * RE];
+  float4 w0[CQ], w1[CQ];
+  auto load = [&](float2 (&xv)[3 * RE], float4 (&wv)[CQ]) {
+#pragma unroll
+    for (int h = 0; h < CQ; ++h) wv[h] = *reinterpret_cast<const float4 *>(w + 4 * Cfg::CG * h);
+    if constexpr (RE == 2) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const float4 v = *reinterpret_cast<const float4 *>(x + 4 * i);
+        xv[2 * i] = make_float2(v.x, v.y), xv[2 * i + 1] = make_float2(v.z, v.w);
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) xv[i] = *reinterpret_cast<const float2 *>(x + 2 * i);
+    }
+    w += Cfg::WS;
+    x += Cfg::RS;
+  };
+  auto product = [&](const float2 (&xv)[3 * RE], const float4 (&wv)[CQ]) {
+#pragma unroll
+    for (int n = 0; n < 4 * CQ; ++n) {
+      const float4 q = wv[n / 4];
+      const float wn = n % 4 == 0 ? q.x : n % 4 == 1 ? q.y : n % 4 == 2 ? q.z : q.w;
+#pragma unroll
+      for (int p = 0; p < 3 * RE; ++p) acc[p][n] = f2fma(xv[p], f2(wn), acc[p][n]);
+    }
+  };
+  load(x0, w0);
+#pragma unroll 1
+  for (int k = 2; k < kc; k += 2) {
+    load(x1, w1);
+    product(x0, w0);
+    load(x0, w0);
+    product(x1, w1);
+  }
+  load(x1, w1);
+  product(x0, w0);
+  product(x1, w1);
+}
+
+// One tile of ne <= EB elements starting at k0 (all threads of the block call it).
+template <int N, int MODE, class Cfg, bool COHERENT>
+__device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, int ne, uint8_t *smem) {
+  using D = Dims<N>;
+  constexpr int NP = D::NP, NFP = D::NFP, NPP = D::NPP, NQ = D::NQ, QC = Cfg::QC, FR = Cfg::FR, NT = Cfg::NT;
+  constexpr int RS = Cfg::RS, CG = Cfg::CG, RE = Cfg::S::RE, CQ = Cfg::S::CQ;
+  float *s_x = reinterpret_cast<float *>(smem), *s_w = reinterpret_cast<float *>(smem + Cfg::OFF_W); // [XR][RS], [XR][WS]
+  float4 *s_fgeo = reinterpret_cast<float4 *>(smem + Cfg::OFF_FGEO);
+  float4 *s_fmat = reinterpret_cast<float4 *>(smem + Cfg::OFF_FMAT);
+  int2 *s_fconn = reinterpret_cast<int2 *>(smem + Cfg::OFF_FCONN);
+  float *s_g = reinterpret_cast<float *>(smem + Cfg::OFF_G); // [EB][GS]
+  float *s_ref = reinterpret_cast<float *>(smem + Cfg::OFF_REF); // [EB][6]
+  const uint8_t *s_fm = smem + Cfg::OFF_TAB, *s_nb = s_fm + D::NFF;
   const int tid = threadIdx.x;
   const int64_t KN = a.K * NPP;
+  const float *u0 = a.u + k0 * NPP;
 
-  for (int idx = tid; idx < 6 * EB * NQ; idx += NT) {
-    int c = idx / (EB * NQ), rem = idx - c * (EB * NQ);
-    int e = rem / NQ, q = rem - e * NQ;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (k0 + e < a.K) v = load_field4<COHERENT>(a.u + c * KN + (k0 + e) * NPP + 4 * q);
-    reinterpret_cast<float4 *>(s_u)[(c * EB + e) * NQ + q] = v;
+  simt_stage_operator<Cfg>(s_w, a.LT, FR < D::NFF ? FR : D::NFF);
+  for (int i = tid; i < ne * 4; i += NT) {
+    cp_async<16>(s_fgeo + i, a.fgeo + k0 * 4 + i);
+    cp_async<16>(s_fmat + i, a.fmat + k0 * 4 + i);
+    cp_async<8>(s_fconn + i, a.fconn + k0 * 4 + i);
   }
-  for (int idx = tid; idx < NFF + kConnKinds * NFP; idx += NT)
-    s_fm[idx] = idx < NFF ? a.fmask[idx] : a.nbrtab[idx - NFF];
+  for (int i = tid; i < 3 * ne; i += NT) {
+    const int e = i / 3, t = i - e * 3;
+    cp_async<16>(s_g + e * Cfg::GS + 4 * t, a.geo + (k0 + e) * G_STRIDE + 4 * t);
+  }
+  // the tile's fields (and residual), on their way to L2
+  for (int c = 0; c < 6; ++c)
+    for (int i = tid * 32; i < ne * NPP; i += NT * 32) {
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(u0 + c * KN + i));
+      if (MODE != MODE_RHS && a.rk_a != 0.f) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.res + c * KN + k0 * NPP + i));
+    }
+  // each field's value at the element's first node (see the volume term)
+  for (int i = tid; i < 6 * ne; i += NT) s_ref[i] = __ldcg(u0 + (i % 6) * KN + (i / 6) * NPP);
+  cp_async_wait();
   __syncthreads();
 
-  const int e = tid / NQ, q = tid - (tid / NQ) * NQ;
-  const bool owner = tid < EB * NQ;
-  const int64_t k = k0 + (owner ? e : 0);
-  const bool live = owner && k < a.K;
-  float vol[6][4];
+  // element group and column group of this thread: neighbouring lanes share the
+  // column group (a 16-byte shared-memory load takes two cycles where lanes l
+  // and l ^ 1 read one address, four to six otherwise)
+  const int rg = (tid >> 1) / CG * 2 + (tid & 1), cg = (tid >> 1) % CG;
+  const bool worker = RE * rg < ne && RE * rg < Cfg::EB;
+  const float *xr = s_x + 6 * RE * rg, *wr = s_w + 4 * cg;
+  float2 acc[3 * RE][4 * CQ];
+#pragma unroll
+  for (int p = 0; p < 3 * RE; ++p)
+#pragma unroll
+    for (int n = 0; n < 4 * CQ; ++n) acc[p][n] = make_float2(0.f, 0.f);
 
-  // ---- local differentiation + chain rule + curl
-  if (owner) {
-    float acc[3][6][4];
+  // ---- flux gather and lifting, FR face nodes of every element at a time:
+  // both traces from L2, the mirror state on walls; upwind flux with the
+  // face's weights. The loads of B face nodes are in flight together.
+#pragma unroll 1
+  for (int r0 = 0; r0 < D::NFF; r0 += FR) {
+    if (r0) __syncthreads(); // the previous product has read X and the operator rows
+    const int fr = D::NFF % FR == 0 || D::NFF - r0 >= FR ? FR : D::NFF - r0;
+    if (r0) simt_stage_operator<Cfg>(s_w, a.LT + r0 * NPP, fr);
+    const int items = ne * FR;
+    constexpr int B = 2;
+#pragma unroll 1
+    for (int it0 = tid; it0 < items; it0 += B * NT) {
+      float qm[B][6], qp[B][6];
+      bool wall[B];
 #pragma unroll
-    for (int d = 0; d < 3; ++d)
+      for (int i = 0; i < B; ++i) {
+        const int it = it0 + i * NT, e = it / FR, r = it - e * FR, fm = r0 + r, f = fm / NFP;
+        wall[i] = false;
+        if (it < items && (D::NFF % FR == 0 || r < fr)) {
+          const int2 cn = s_fconn[e * 4 + f];
+          const float *um = u0 + e * NPP + s_fm[fm], *up = um;
+          wall[i] = cn.y == kBoundaryConn;
+          if (!wall[i]) up = a.u + int64_t(cn.x) * NPP + s_nb[cn.y * NFP + fm - f * NFP];
 #pragma unroll
-      for (int c = 0; c < 6; ++c)
+          for (int c = 0; c < 6; ++c) qm[i][c] = load_trace<COHERENT>(um + c * KN);
 #pragma unroll
-        for (int n = 0; n < 4; ++n) acc[d][c][n] = 0.f;
-    const float *su = s_u + e * NPP;
-#pragma unroll 2
-    for (int j = 0; j < NP; ++j) {
-      float4 dr = ldg4(a.DT + (0 * NP + j) * NPP + 4 * q);
-      float4 ds = ldg4(a.DT + (1 * NP + j) * NPP + 4 * q);
-      float4 dt = ldg4(a.DT + (2 * NP + j) * NPP + 4 * q);
-      const float dv[3][4] = {{dr.x, dr.y, dr.z, dr.w}, {ds.x, ds.y, ds.z, ds.w}, {dt.x, dt.y, dt.z, dt.w}};
-#pragma unroll
-      for (int c = 0; c < 6; ++c) {
-        float uj = su[c * EB * NPP + j];
-        // packed FP32 pairs: two output nodes per instruction
-#pragma unroll
-        for (int d = 0; d < 3; ++d)
-#pragma unroll
-          for (int n = 0; n < 4; n += 2) {
-            const float2 r = f2fma(make_float2(dv[d][n], dv[d][n + 1]), f2(uj), make_float2(acc[d][c][n], acc[d][c][n + 1]));
-            acc[d][c][n] = r.x;
-            acc[d][c][n + 1] = r.y;
-          }
-      }
-    }
-    const float *g = a.geo + (live ? k : 0) * G_STRIDE;
-    float m[9];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) m[i] = __ldg(g + i);
-    // m = {rx ry rz sx sy sz tx ty tz}: d/dx_l = m[l] d/dr + m[3+l] d/ds + m[6+l] d/dt
-#pragma unroll
-    for (int n = 0; n < 4; ++n) {
-      float dd[6][3];
-#pragma unroll
-      for (int c = 0; c < 6; ++c)
-#pragma unroll
-        for (int l = 0; l < 3; ++l) dd[c][l] = m[l] * acc[0][c][n] + m[3 + l] * acc[1][c][n] + m[6 + l] * acc[2][c][n];
-      vol[0][n] = dd[5][1] - dd[4][2];    // (curl H)_x
-      vol[1][n] = dd[3][2] - dd[5][0];    // (curl H)_y
-      vol[2][n] = dd[4][0] - dd[3][1];    // (curl H)_z
-      vol[3][n] = -(dd[2][1] - dd[1][2]); // -(curl E)_x
-      vol[4][n] = -(dd[0][2] - dd[2][0]); // -(curl E)_y
-      vol[5][n] = -(dd[1][0] - dd[0][1]); // -(curl E)_z
-    }
-  }
-
-  // ---- flux gather
-  for (int it = tid; it < EB * NFF; it += NT) {
-    int ee = it / NFF, fm = it - ee * NFF;
-    int f = fm / NFP, mm = fm - f * NFP;
-    int64_t kk = k0 + ee;
-    float fl[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (kk < a.K) {
-      int vm = s_fm[fm];
-      float qm[6], qp[6];
-#pragma unroll
-      for (int c = 0; c < 6; ++c) qm[c] = s_u[(c * EB + ee) * NPP + vm];
-      const int2 cn = __ldg(a.fconn + kk * 4 + f);
-      const float4 nf = __ldg(a.fgeo + kk * 4 + f);
-      const float4 wf = __ldg(a.fmat + kk * 4 + f); // face weights (neighbour or mirror impedances)
-      if (cn.y == kBoundaryConn) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          qp[c] = -qm[c];
-          qp[c + 3] = qm[c + 3];
+          for (int c = 0; c < 6; ++c) qp[i][c] = load_trace<COHERENT>(up + c * KN);
         }
-      } else {
-        int vn = s_nb[cn.y * NFP + mm];
-        const float *up = a.u + int64_t(cn.x) * NPP + vn;
-#pragma unroll
-        for (int c = 0; c < 6; ++c) qp[c] = load_field<COHERENT>(up + c * KN);
       }
-      maxwell_flux_w(nf, qm, qp, wf, a.alpha, fl);
-    }
 #pragma unroll
-    for (int c = 0; c < 6; ++c) s_fl[(c * EB + ee) * NFF + fm] = fl[c];
+      for (int i = 0; i < B; ++i) {
+        const int it = it0 + i * NT, e = it / FR, r = it - e * FR, fm = r0 + r, f = fm / NFP;
+        if (it >= items || (D::NFF % FR != 0 && r >= fr)) break;
+        if (wall[i]) {
+#pragma unroll
+          for (int c = 0; c < 3; ++c) qp[i][c] = -qm[i][c];
+        }
+        float fl[6];
+        maxwell_flux_w(s_fgeo[e * 4 + f], qm[i], qp[i], s_fmat[e * 4 + f], a.alpha, fl);
+        float2 *d = reinterpret_cast<float2 *>(s_x + r * RS + e * 6);
+        d[0] = make_float2(fl[0], fl[1]);
+        d[1] = make_float2(fl[2], fl[3]);
+        d[2] = make_float2(fl[4], fl[5]);
+      }
+    }
+    cp_async_wait();
+    __syncthreads();
+    if (worker) simt_product<Cfg>(acc, xr, wr, fr);
   }
-  __syncthreads();
 
-  if (!owner) return;
-  // ---- flux lifting
-  {
-    const float *sf = s_fl + e * NFF;
-#pragma unroll 4
-    for (int fm = 0; fm < NFF; ++fm) {
-      float4 L = ldg4(a.LT + fm * NPP + 4 * q);
+  // ---- volume term, QC node quads at a time: the combinations of the curl
+  // (d/dx_l = sum_d (dr_d/dx_l) d/dr_d) of every node and direction, then
+  // their derivatives. The fields enter as differences from their value at the
+  // element's first node: D annihilates constants, and without the constant
+  // part neither the rounded combinations nor the sums carry its rounding
+  // error (right-hand side at N=5 against 64 bits: 1.5e-6 with it, 9.5e-7
+  // without; 8.7e-7 with the combinations taken after the differentiation).
+#pragma unroll 1
+  for (int q0 = 0; q0 < NQ; q0 += QC) {
+    __syncthreads(); // the previous product has read X and the operator rows
+    const int qn = NQ - q0 < QC ? NQ - q0 : QC;
+    simt_stage_operator<Cfg>(s_w, a.DT + 12 * q0 * NPP, 12 * qn);
+    for (int it = tid; it < ne * QC; it += NT) {
+      const int e = it / QC, qq = it - e * QC;
+      if (qq >= qn) continue;
+      const float *up = u0 + e * NPP + 4 * (q0 + qq);
+      float4 v4[6];
+#pragma unroll
+      for (int c = 0; c < 6; ++c) v4[c] = load_field4(up + c * KN);
+      float v[6][4];
 #pragma unroll
       for (int c = 0; c < 6; ++c) {
-        float gv = sf[c * EB * NFF + fm];
-        const float2 v01 = f2fma(make_float2(L.x, L.y), f2(gv), make_float2(vol[c][0], vol[c][1]));
-        const float2 v23 = f2fma(make_float2(L.z, L.w), f2(gv), make_float2(vol[c][2], vol[c][3]));
-        vol[c][0] = v01.x, vol[c][1] = v01.y, vol[c][2] = v23.x, vol[c][3] = v23.y;
+        const float r = s_ref[e * 6 + c];
+        v[c][0] = v4[c].x - r, v[c][1] = v4[c].y - r, v[c][2] = v4[c].z - r, v[c][3] = v4[c].w - r;
+        if (NP % 4 != 0 && q0 + qq == NQ - 1) { // padding entries are ignored
+#pragma unroll
+          for (int n = NP % 4; n < 4; ++n) v[c][n] = 0.f;
+        }
+      }
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const float gx = s_g[e * Cfg::GS + 3 * d], gy = s_g[e * Cfg::GS + 3 * d + 1], gz = s_g[e * Cfg::GS + 3 * d + 2];
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+          const float Ex = v[0][n], Ey = v[1][n], Ez = v[2][n], Hx = v[3][n], Hy = v[4][n], Hz = v[5][n];
+          float2 *x = reinterpret_cast<float2 *>(s_x + (3 * (4 * qq + n) + d) * RS + e * 6);
+          x[0] = make_float2(gy * Hz - gz * Hy, gz * Hx - gx * Hz); // curl H
+          x[1] = make_float2(gx * Hy - gy * Hx, gz * Ey - gy * Ez); //         , -curl E
+          x[2] = make_float2(gx * Ez - gz * Ex, gy * Ex - gx * Ey);
+        }
       }
     }
+    cp_async_wait();
+    __syncthreads();
+    if (worker) simt_product<Cfg>(acc, xr, wr, 12 * qn);
   }
-  if (!live) return;
-  // ---- material scaling and output / operator assembly
-  const float ie = __ldg(a.geo + k * G_STRIDE + G_IEPS), im = __ldg(a.geo + k * G_STRIDE + G_IMU);
-  const float dtk = a.dt_geo ? __ldg(a.geo + k * G_STRIDE + G_DT) : a.dt;
+
+  // ---- material scaling and output / operator assembly, three fields of an
+  // element and node quad at a time (their loads in flight together)
+  if (!worker) return;
 #pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    const float w = c < 3 ? ie : im;
-    float r4[4];
+  for (int bt = 0; bt < 2 * RE * CQ; ++bt) { // (element of the group, E or H, quad)
+    const int el = bt / (2 * CQ), g = bt / CQ % 2, h = bt % CQ, e = RE * rg + el, q = cg + h * CG;
+    if (e >= ne || q >= NQ) continue;
+    const float *geo = a.geo + (k0 + e) * G_STRIDE;
+    const float w = __ldg(geo + (g ? G_IMU : G_IEPS)), dtk = a.dt_geo ? __ldg(geo + G_DT) : a.dt;
+    const int64_t off0 = 3 * g * KN + (k0 + e) * NPP + 4 * q;
+    float4 rs[3], uo[3];
+    if (MODE != MODE_RHS) {
 #pragma unroll
-    for (int n = 0; n < 4; ++n) r4[n] = (4 * q + n < NP) ? vol[c][n] * w : 0.f;
-    const int64_t off = c * KN + k * NPP + 4 * q;
-    if (MODE == MODE_RHS) {
-      *reinterpret_cast<float4 *>(a.rhs + off) = make_float4(r4[0], r4[1], r4[2], r4[3]);
-    } else {
-      // the first LSERK4 stage has a = 0: the residual it overwrites is not read
-      float4 rs = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (a.rk_a != 0.f)
-        rs = COHERENT ? __ldcg(reinterpret_cast<const float4 *>(a.res + off))
-                      : *reinterpret_cast<const float4 *>(a.res + off);
-      float4 uo = reinterpret_cast<const float4 *>(s_u)[(c * EB + e) * NQ + q];
-      float rv[4] = {rs.x, rs.y, rs.z, rs.w}, uv[4] = {uo.x, uo.y, uo.z, uo.w};
+      for (int c = 0; c < 3; ++c) {
+        // the first LSERK4 stage has a = 0: the residual it overwrites is not read
+        rs[c] = a.rk_a != 0.f ? load_field4(a.res + c * KN + off0) : make_float4(0.f, 0.f, 0.f, 0.f);
+        uo[c] = load_field4(a.u + c * KN + off0);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const int64_t off = c * KN + off0;
+      const int row = 6 * el + 3 * g + c;
+      float r4[4];
 #pragma unroll
       for (int n = 0; n < 4; ++n) {
-        bool pad = 4 * q + n >= NP;
-        rv[n] = pad ? 0.f : fmaf(a.rk_a, rv[n], dtk * r4[n]);
-        uv[n] = pad ? 0.f : fmaf(a.rk_b, rv[n], uv[n]);
+        const float2 v = acc[row / 2][4 * h + n];
+        r4[n] = (4 * q + n < NP) ? (row % 2 ? v.y : v.x) * w : 0.f;
       }
-      *reinterpret_cast<float4 *>(a.res + off) = make_float4(rv[0], rv[1], rv[2], rv[3]);
-      *reinterpret_cast<float4 *>(a.u_out + off) = make_float4(uv[0], uv[1], uv[2], uv[3]);
-      // the adjoint's eps gradient reads only the E components of the stage right-hand side
-      if (MODE == MODE_LSERK_STORE && c < 3)
+      if (MODE == MODE_RHS) {
         *reinterpret_cast<float4 *>(a.rhs + off) = make_float4(r4[0], r4[1], r4[2], r4[3]);
+      } else {
+        float rv[4] = {rs[c].x, rs[c].y, rs[c].z, rs[c].w}, uv[4] = {uo[c].x, uo[c].y, uo[c].z, uo[c].w};
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+          const bool pad = 4 * q + n >= NP;
+          rv[n] = pad ? 0.f : fmaf(a.rk_a, rv[n], dtk * r4[n]);
+          uv[n] = pad ? 0.f : fmaf(a.rk_b, rv[n], uv[n]);
+        }
+        *reinterpret_cast<float4 *>(a.res + off) = make_float4(rv[0], rv[1], rv[2], rv[3]);
+        *reinterpret_cast<float4 *>(a.u_out + off) = make_float4(uv[0], uv[1], uv[2], uv[3]);
+        // the adjoint's eps gradient reads only the E components of the stage right-hand side
+        if (MODE == MODE_LSERK_STORE && g == 0)
+          *reinterpret_cast<float4 *>(a.rhs + off) = make_float4(r4[0], r4[1], r4[2], r4[3]);
+      }
     }
   }
 }
 
-template <int N, int MODE>
-__global__ void __launch_bounds__(SimtCfg<N>::NT) k_stage_simt(StageArgs a) {
+template <int N, int MODE, bool SMALL>
+__global__ void __launch_bounds__(SimtCfg<N, SMALL>::NT, SimtCfg<N, SMALL>::MINB) k_stage_simt(StageArgs a, TileMap tm) {
+  using Cfg = SimtCfg<N, SMALL>;
   extern __shared__ float4 smem4[];
-  constexpr int EB = SimtCfg<N>::EB;
-  const int64_t ntiles = (a.K + EB - 1) / EB;
+  simt_setup<Cfg>(a, smem4);
   pdl_wait(); // stage after stage: fields of the previous stage from here on
-  for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    if (t + int64_t(gridDim.x) >= ntiles) pdl_launch_next(); // this block's last tile
-    __syncthreads(); // shared memory of the previous tile is no longer read
-    simt_stage_tile<N, MODE, EB, true>(a, t * EB, smem4);
+  for (int t = blockIdx.x; t < tm.ntiles; t += gridDim.x) {
+    if (t + int(gridDim.x) >= tm.ntiles) pdl_launch_next(); // this block's last tile
+    if (t != int(blockIdx.x)) __syncthreads(); // shared memory of the previous tile is no longer read
+    simt_stage_tile<N, MODE, Cfg, false>(a, tm.start(t), tm.size(t, a.K), reinterpret_cast<uint8_t *>(smem4));
   }
 }
 
-template <int N>
-cudaError_t launch_simt_order(int mode, const StageArgs &a, cudaStream_t s) {
-  using Cfg = SimtCfg<N>;
-  const void *kern = mode == MODE_RHS ? (const void *)k_stage_simt<N, MODE_RHS>
-                     : mode == MODE_LSERK ? (const void *)k_stage_simt<N, MODE_LSERK>
-                                          : (const void *)k_stage_simt<N, MODE_LSERK_STORE>;
+template <int N, int MODE, bool SMALL>
+cudaError_t launch_simt_mode(const StageArgs &a, int dev, int sms, cudaStream_t s) {
+  using Cfg = SimtCfg<N, SMALL>;
+  auto kern = k_stage_simt<N, MODE, SMALL>;
   // the shared-memory opt-in is a per-device function attribute: set it on every launch
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Cfg::SMEM));
-  int dev = 0, sms = 0;
-  if (e == cudaSuccess) e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   // persistent grid: as many blocks as fit on the GPU at once (at most one per
   // tile); blocks per SM of each kernel cached per device
   constexpr int kDevCache = 64;
-  static std::atomic<int> per_sm_cache[3][kDevCache];
-  int per_sm = dev < kDevCache ? per_sm_cache[mode][dev].load(std::memory_order_relaxed) : 0;
+  static std::atomic<int> per_sm_cache[kDevCache];
+  int per_sm = dev < kDevCache ? per_sm_cache[dev].load(std::memory_order_relaxed) : 0;
   if (per_sm == 0) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, Cfg::NT, Cfg::SMEM);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    if (dev < kDevCache) per_sm_cache[mode][dev].store(per_sm, std::memory_order_relaxed);
+    if (dev < kDevCache) per_sm_cache[dev].store(per_sm, std::memory_order_relaxed);
   }
-  const int64_t ntiles = (a.K + Cfg::EB - 1) / Cfg::EB, cap = int64_t(per_sm) * sms;
-  const unsigned blocks = unsigned(ntiles < cap ? ntiles : cap);
-  if (mode == MODE_RHS) return launch_pdl(k_stage_simt<N, MODE_RHS>, dim3(blocks), dim3(Cfg::NT), Cfg::SMEM, s, a);
-  if (mode == MODE_LSERK) return launch_pdl(k_stage_simt<N, MODE_LSERK>, dim3(blocks), dim3(Cfg::NT), Cfg::SMEM, s, a);
-  return launch_pdl(k_stage_simt<N, MODE_LSERK_STORE>, dim3(blocks), dim3(Cfg::NT), Cfg::SMEM, s, a);
+  const TileMap tm = make_tiles(a.K, per_sm * sms, Cfg::EB);
+  const unsigned blocks = unsigned(tm.ntiles < per_sm * sms ? tm.ntiles : per_sm * sms);
+  return launch_pdl(kern, dim3(blocks), dim3(Cfg::NT), Cfg::SMEM, s, a, tm);
+}
+
+// The two-element shape runs in rounds of one tile per block that take the same
+// time however many elements a tile has; the small shape's time grows with the
+// element count, by simt_round_ratio times a round's time per full round of
+// elements (measured, us per round and us per full round's elements in the
+// small shape: N=4 50 / 61, N=5 63 / 85, N=7 103 / 128, N=8 134 / 181, N=9 168 /
+// 228). The first is taken where its rounds cost less.
+template <int N>
+constexpr double simt_round_ratio() {
+  return N == 4 ? 1.22 : N == 7 ? 1.24 : 1.35;
+}
+template <int N>
+bool simt_small(int64_t K, int sms) {
+  if (simt_small_only<N>()) return true;
+  const double rounds = double(K) / (double(SimtCfg<N, false>::MINB) * sms * SimtShape<N, false>::EB);
+  return std::ceil(rounds) >= simt_round_ratio<N>() * rounds;
+}
+
+template <int N, int MODE>
+cudaError_t launch_simt_shape(const StageArgs &a, cudaStream_t s) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  if constexpr (!simt_small_only<N>())
+    if (!simt_small<N>(a.K, sms)) return launch_simt_mode<N, MODE, false>(a, dev, sms, s);
+  return launch_simt_mode<N, MODE, true>(a, dev, sms, s);
+}
+
+template <int N>
+cudaError_t launch_simt_order(int mode, const StageArgs &a, cudaStream_t s) {
+  if (mode == MODE_RHS) return launch_simt_shape<N, MODE_RHS>(a, s);
+  if (mode == MODE_LSERK) return launch_simt_shape<N, MODE_LSERK>(a, s);
+  return launch_simt_shape<N, MODE_LSERK_STORE>(a, s);
 }
 
 } // namespace dgmx

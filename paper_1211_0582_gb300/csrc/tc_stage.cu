@@ -43,6 +43,7 @@
 #include "grid_sync.cuh"
 #include "tc_api.h"
 #include "tc_common.cuh"
+#include "tiles.cuh"
 #include "umma.cuh"
 
 namespace dgmx {
@@ -54,30 +55,6 @@ using namespace tcc;
 constexpr int kThreads = 512;
 constexpr int kTileElems = 20; // 4 TMEM lane quarters x 5 elements
 
-// Element ranges of the tiles: whole rounds of full tiles (kTileElems elements,
-// `grid` tiles per round), then the remaining elements in tiles of `small`
-// elements, sized so that the last round spreads over the whole grid instead
-// of leaving most CTAs idle behind a few full tiles.
-struct TileMap {
-  int nfull, small, ntiles;
-  __host__ __device__ int64_t start(int t) const {
-    return t < nfull ? int64_t(t) * kTileElems : int64_t(nfull) * kTileElems + int64_t(t - nfull) * small;
-  }
-  __host__ __device__ int size(int t, int64_t K) const {
-    const int64_t k0 = start(t), n = t < nfull ? kTileElems : small;
-    return int(K - k0 < n ? K - k0 : n);
-  }
-};
-
-TileMap make_tiles(int64_t K, int grid) {
-  const int64_t nfull = K / kTileElems / grid * grid;
-  const int64_t rest = K - nfull * kTileElems;
-  int64_t small = (rest + grid - 1) / grid;
-  if (small < 1) small = 1;
-  if (small > kTileElems) small = kTileElems;
-  const int64_t nsmall = (rest + small - 1) / small;
-  return TileMap{int(nfull), int(small), int(nfull + nsmall)};
-}
 constexpr int kMaxTcOrder = 7; // N <= 5 here, N = 6, 7 in tc_stage_streamed.cu
 
 template <int N>
@@ -1501,7 +1478,7 @@ cudaError_t launch_tc_kernel(const StageArgs &a, const TcState &st, int *flag, c
   auto kern = k_stage_tc<N, MODE, BF16, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM);
   if (e != cudaSuccess) return e;
-  const TileMap tm = make_tiles(a.K, st.sms);
+  const TileMap tm = make_tiles(a.K, st.sms, kTileElems);
   const int grid = tm.ntiles < st.sms ? tm.ntiles : st.sms;
   return launch_pdl(kern, dim3(unsigned(grid)), dim3(kThreads), size_t(T::SMEM), s, a,
                     reinterpret_cast<const uint4 *>(st.d_ops), tm, flag, EnsLaunch{});
@@ -1513,7 +1490,7 @@ cudaError_t launch_tcw_kernel(const StageArgs &a, const TcState &st, int *flag, 
   auto kern = k_stage_tcw<N, MODE, BF16>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM);
   if (e != cudaSuccess) return e;
-  const TileMap tm = make_tiles(a.K, st.sms);
+  const TileMap tm = make_tiles(a.K, st.sms, kTileElems);
   const int grid = tm.ntiles < st.sms ? tm.ntiles : st.sms;
   return launch_pdl(kern, dim3(unsigned(grid)), dim3(kWsThreads), size_t(L::SMEM), s, a,
                     reinterpret_cast<const uint4 *>(st.d_ops), tm, flag);
@@ -1527,7 +1504,7 @@ cudaError_t launch_tc_ens_kernel(const StageArgs &a, const TcState &st, const En
   auto kern = k_stage_tc<N, MODE_LSERK, BF16, true>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM);
   if (e != cudaSuccess) return e;
-  const TileMap tm = make_tiles(a.K, st.sms);
+  const TileMap tm = make_tiles(a.K, st.sms, kTileElems);
   const int grid = tm.ntiles < st.sms ? tm.ntiles : st.sms;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(unsigned(grid));
