@@ -18,7 +18,7 @@ namespace dgmx {
 template <int N, class Cfg>
 __global__ void __launch_bounds__(Cfg::NT, Cfg::MINB)
     k_ensemble_persistent(StageArgs a, StageCoeffs rk, float *u_a, float *u_b, int nsteps, GridBarrier *gb,
-                          TileMap tm, int *err_flag) {
+                          TileMap<Cfg::EB> tm, int *err_flag) {
   extern __shared__ float4 smem4[];
   uint8_t *smem = reinterpret_cast<uint8_t *>(smem4);
   bool flip = false;
@@ -76,7 +76,7 @@ cudaError_t launch_ensemble_cfg(const StageArgs &a, const StageCoeffs &rk, float
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   if (occ == 1) per_sm = (per_sm + 1) / 2;
   if (used) *used = per_sm;
-  const TileMap tm = make_tiles(a.K, per_sm * sms, Cfg::EB);
+  const TileMap<Cfg::EB> tm = make_tiles<Cfg::EB>(a.K, per_sm * sms);
   const unsigned grid = unsigned(tm.ntiles < per_sm * sms ? tm.ntiles : per_sm * sms);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid);

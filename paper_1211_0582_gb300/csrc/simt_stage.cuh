@@ -382,7 +382,7 @@ __device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, 
 }
 
 template <int N, int MODE, bool SMALL>
-__global__ void __launch_bounds__(SimtCfg<N, SMALL>::NT, SimtCfg<N, SMALL>::MINB) k_stage_simt(StageArgs a, TileMap tm) {
+__global__ void __launch_bounds__(SimtCfg<N, SMALL>::NT, SimtCfg<N, SMALL>::MINB) k_stage_simt(StageArgs a, TileMap<SimtCfg<N, SMALL>::EB> tm) {
   using Cfg = SimtCfg<N, SMALL>;
   extern __shared__ float4 smem4[];
   simt_setup<Cfg>(a, smem4);
@@ -412,7 +412,7 @@ cudaError_t launch_simt_mode(const StageArgs &a, int dev, int sms, cudaStream_t 
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     if (dev < kDevCache) per_sm_cache[dev].store(per_sm, std::memory_order_relaxed);
   }
-  const TileMap tm = make_tiles(a.K, per_sm * sms, Cfg::EB);
+  const TileMap<Cfg::EB> tm = make_tiles<Cfg::EB>(a.K, per_sm * sms);
   const unsigned blocks = unsigned(tm.ntiles < per_sm * sms ? tm.ntiles : per_sm * sms);
   return launch_pdl(kern, dim3(blocks), dim3(Cfg::NT), Cfg::SMEM, s, a, tm);
 }

@@ -52,7 +52,6 @@ namespace {
 
 using namespace tcc;
 
-constexpr int kThreads = 512;
 constexpr int kTileElems = 20; // 4 TMEM lane quarters x 5 elements
 
 constexpr int kMaxTcOrder = 7; // N <= 5 here, N = 6, 7 in tc_stage_streamed.cu
@@ -71,7 +70,8 @@ struct TC {
   static constexpr int CU = CA + K1;           // TMEM columns of the tile's fields (FP32) for the update
   static constexpr int TCOLS = tmem_cols(CU + K1);
   static_assert(CU + K1 <= 512, "accumulators, the A1 operand and the fields exceed tensor memory");
-  static_assert(K1 <= 16 * (kThreads / 128), "the field split covers 16 K values per warp, four warps per quarter");
+  static constexpr int THREADS = N <= 3 ? 256 : 512; // per block of the single-tile kernel
+  static_assert(K1 <= 16 * (THREADS / 128), "the field split covers 16 K values per warp, THREADS / 128 warps per quarter");
   static constexpr int FS = kTileElems * NPP + 4; // padded field-block stride of the staged tiles
   // A2 in the K-major core-matrix layout with padded strides: 144 bytes
   // between the core matrices of a row group along K (not 128) and a row-group
@@ -116,6 +116,16 @@ struct TC {
   static constexpr int OFF_MX = OFF_TAB + rup(NFF + kConnKinds * NFP, 16);
   static constexpr int OFF_BAR = OFF_MX + 128 * 4 + 2 * kTileElems * 4 + 128 * 4; // mbarriers: GEMM1, GEMM2, residual, next tile; TMEM slot
   static constexpr int SMEM = OFF_BAR + 48;
+  // Blocks per SM of a single-stage launch. One tile's phases are a chain of
+  // latencies; where a tile, the operators and the tensor memory columns of
+  // several blocks fit, the other blocks' tiles fill the gaps, and half the
+  // threads per block keep their registers. Two blocks at N = 4 would need
+  // 2 x 137 KB of shared memory. At N = 2 four blocks are faster on large meshes
+  // (80 us) but slower below 5,000 elements. Measured (FP16x3, us per stage, one
+  // block of 512 threads and now): N=1 162,000 tets 125 -> 55; N=2 131,712 tets
+  // 134 -> 89; N=3 131,712 tets 161 -> 115 (two blocks of 512 threads: 133).
+  static constexpr int BLOCKS = N == 1 ? 4 : N <= 3 ? 2 : 1;
+  static_assert(BLOCKS * TCOLS <= 512 && BLOCKS * (SMEM + 1024) <= 228 * 1024, "BLOCKS per SM do not fit");
 };
 
 // Three split products per K step: hi*hi, hi*lo, lo*hi, FP32 accumulation.
@@ -181,10 +191,11 @@ __device__ uint32_t g_tc_trace[kTraceBlocks * kTraceTiles * kTcEvents];
 // stage (a stage reads the neighbours' states the previous one wrote), field
 // gathers through L2 (another SM's L1 may hold a copy from two stages ago).
 template <int N, int MODE, bool BF16, bool ENS>
-__global__ void __launch_bounds__(kThreads, 1)
-    k_stage_tc(StageArgs a, const uint4 *__restrict__ ops, TileMap tm, int *err_flag, EnsLaunch ens) {
+__global__ void __launch_bounds__(ENS ? 512 : TC<N>::THREADS, ENS ? 1 : TC<N>::BLOCKS)
+    k_stage_tc(StageArgs a, const uint4 *__restrict__ ops, TileMap<kTileElems> tm, int *err_flag, EnsLaunch ens) {
   using T = TC<N>;
   constexpr int NP = T::NP, NFP = T::NFP, NPP = T::NPP, NFF = T::NFF, FS = T::FS;
+  constexpr int NTH = ENS ? 512 : T::THREADS, NW = NTH / 32; // threads, warps
   extern __shared__ __align__(1024) uint8_t smem[];
   float *s_ub = reinterpret_cast<float *>(smem + T::OFF_U);      // [2][6][FS]: fields by tile parity
   float *s_res = reinterpret_cast<float *>(smem + T::OFF_RES);   // [6][FS]: residual of the tile
@@ -205,10 +216,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   // single-thread roles sit in the last four warps, which have the least flux
   // and epilogue work (issuing a tcgen05.mma or a bulk copy stalls the thread):
   // MMA issue, staging of the next tile, residual load, bulk stores
-  const bool issuer = tid == kThreads - 32;
-  const bool stager = tid == kThreads - 64;
-  const bool rloader = tid == kThreads - 96;
-  const bool storer = tid == kThreads - 128;
+  const bool issuer = tid == NTH - 32;
+  const bool stager = tid == NTH - 64;
+  const bool rloader = tid == NTH - 96;
+  const bool storer = tid == NTH - 128;
   const int64_t KN = a.K * NPP;
   const uint32_t sbase = umma::smem_u32(smem);
   const long long wlim = umma::wait_cycles(a.wait_limit); // main waits; drains use the default
@@ -232,13 +243,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   };
 
   // ---- one-time setup
-  for (int i = tid; i < T::A2R / 16; i += kThreads)
+  for (int i = tid; i < T::A2R / 16; i += NTH)
     reinterpret_cast<uint4 *>(smem + T::OFF_A2H)[i] = make_uint4(0u, 0u, 0u, 0u);
-  for (int i = tid; i < T::OPS_BYTES / 16; i += kThreads)
+  for (int i = tid; i < T::OPS_BYTES / 16; i += NTH)
     reinterpret_cast<uint4 *>(smem + T::OFF_B1H)[i] = __ldg(ops + i);
-  for (int i = tid; i < NFF + kConnKinds * NFP; i += kThreads)
+  for (int i = tid; i < NFF + kConnKinds * NFP; i += NTH)
     s_fm[i] = i < NFF ? a.fmask[i] : a.nbrtab[i - NFF];
-  for (int i = tid; i < 256 + 2 * kTileElems; i += kThreads) s_inv1[i] = i < 128 ? 1.f : 0.f;
+  for (int i = tid; i < 256 + 2 * kTileElems; i += NTH) s_inv1[i] = i < 128 ? 1.f : 0.f;
   if (tid == 0) {
     umma::mbar_init(bar1, 1);
     umma::mbar_init(bar2, 1);
@@ -276,11 +287,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   // flux: blocks of 4 elements x 16 columns of A2 (padding columns included,
   // written as zeros), lane -> (element, pair of adjacent columns); column
   // f * NFPE + m holds face node m of face f, so a pair never straddles two
-  // faces; block b goes to warp b % 16, so the last warps get the fewest
+  // faces; block b goes to warp b % NW, so the last warps get the fewest
   constexpr int NFPE = T::NFPE;
   constexpr int KGF = T::K2 / 16;
   constexpr int NBLK = (kTileElems / 4) * KGF;
-  constexpr int R2 = (NBLK + 15) / 16;
+  constexpr int R2 = (NBLK + NW - 1) / NW;
   const int eo = lane >> 3, kp = lane & 7;
   // this lane's own face-node traces in the tile buffer (element row offset
   // plus volume node; the pair's second node falls back to the first past the
@@ -288,7 +299,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   int own_off[R2];
 #pragma unroll
   for (int s = 0; s < R2; ++s) {
-    const int blk = warp + 16 * s;
+    const int blk = warp + NW * s;
     const int e = 4 * (blk / KGF) + eo, fm = 16 * (blk % KGF) + 2 * kp;
     const int f = fm / NFPE, mm = fm - f * NFPE;
     own_off[s] = 0;
@@ -314,7 +325,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int soff = fld * FS + e_loc * NPP; // this lane's row in the staged tiles
   const uint32_t lane_taddr = tmem + (uint32_t(quarter * 32) << 16);
   constexpr int NCH = (NP + 7) / 8;
-  constexpr int CPP = (NCH + 3) / 4;
+  constexpr int CPP = (NCH + NTH / 128 - 1) / (NTH / 128);
   const int ch0 = part * CPP;
   const int ch1 = (part + 1) * CPP < NCH ? (part + 1) * CPP : NCH;
 
@@ -432,7 +443,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       int lidx[R2][2];
 #pragma unroll
       for (int s = 0; s < R2; ++s) {
-        const int blk = warp + 16 * s;
+        const int blk = warp + NW * s;
         const int e = 4 * (blk / KGF) + eo, fm = 16 * (blk % KGF) + 2 * kp;
         const int f = fm / NFPE, mm = fm - f * NFPE;
 #pragma unroll
@@ -465,7 +476,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       float fl[R2][2][6];
 #pragma unroll
       for (int s = 0; s < R2; ++s) {
-        const int blk = warp + 16 * s;
+        const int blk = warp + NW * s;
         const int e = 4 * (blk / KGF) + eo, fm = 16 * (blk % KGF) + 2 * kp;
         const int f = fm / NFPE, mm = fm - f * NFPE;
 #pragma unroll
@@ -574,7 +585,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       {
 #pragma unroll
         for (int s = 0; s < R2; ++s) {
-          const int blk = warp + 16 * s;
+          const int blk = warp + NW * s;
           const int e = 4 * (blk / KGF) + eo, fm = 16 * (blk % KGF) + 2 * kp;
           if (blk < NBLK) {
             float sc2[6];
@@ -863,7 +874,7 @@ struct TW {
 
 template <int N, int MODE, bool BF16>
 __global__ void __launch_bounds__(kWsThreads, 1)
-    k_stage_tcw(StageArgs a, const uint4 *__restrict__ ops, TileMap tm, int *err_flag) {
+    k_stage_tcw(StageArgs a, const uint4 *__restrict__ ops, TileMap<kTileElems> tm, int *err_flag) {
   using T = TC<N>;
   using L = TW<N>;
   constexpr int NP = T::NP, NFP = T::NFP, NPP = T::NPP, NFF = T::NFF, FS = T::FS;
@@ -1477,10 +1488,14 @@ cudaError_t launch_tc_kernel(const StageArgs &a, const TcState &st, int *flag, c
   static_assert(T::SMEM <= 232448, "tensor-core tile does not fit in shared memory");
   auto kern = k_stage_tc<N, MODE, BF16, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM);
+  // the largest shared-memory carveout, so that the blocks of an SM fit side by side
+  if (e == cudaSuccess && T::BLOCKS > 1) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   if (e != cudaSuccess) return e;
-  const TileMap tm = make_tiles(a.K, st.sms, kTileElems);
-  const int grid = tm.ntiles < st.sms ? tm.ntiles : st.sms;
-  return launch_pdl(kern, dim3(unsigned(grid)), dim3(kThreads), size_t(T::SMEM), s, a,
+  // a mesh of at most one tile per SM is spread over the SMs, not over their blocks
+  const int blocks = a.K <= int64_t(kTileElems) * st.sms ? st.sms : T::BLOCKS * st.sms;
+  const TileMap<kTileElems> tm = make_tiles<kTileElems>(a.K, blocks);
+  const int grid = tm.ntiles < blocks ? tm.ntiles : blocks;
+  return launch_pdl(kern, dim3(unsigned(grid)), dim3(T::THREADS), size_t(T::SMEM), s, a,
                     reinterpret_cast<const uint4 *>(st.d_ops), tm, flag, EnsLaunch{});
 }
 
@@ -1490,7 +1505,7 @@ cudaError_t launch_tcw_kernel(const StageArgs &a, const TcState &st, int *flag, 
   auto kern = k_stage_tcw<N, MODE, BF16>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM);
   if (e != cudaSuccess) return e;
-  const TileMap tm = make_tiles(a.K, st.sms, kTileElems);
+  const TileMap<kTileElems> tm = make_tiles<kTileElems>(a.K, st.sms);
   const int grid = tm.ntiles < st.sms ? tm.ntiles : st.sms;
   return launch_pdl(kern, dim3(unsigned(grid)), dim3(kWsThreads), size_t(L::SMEM), s, a,
                     reinterpret_cast<const uint4 *>(st.d_ops), tm, flag);
@@ -1504,11 +1519,11 @@ cudaError_t launch_tc_ens_kernel(const StageArgs &a, const TcState &st, const En
   auto kern = k_stage_tc<N, MODE_LSERK, BF16, true>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM);
   if (e != cudaSuccess) return e;
-  const TileMap tm = make_tiles(a.K, st.sms, kTileElems);
+  const TileMap<kTileElems> tm = make_tiles<kTileElems>(a.K, st.sms);
   const int grid = tm.ntiles < st.sms ? tm.ntiles : st.sms;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(unsigned(grid));
-  cfg.blockDim = dim3(kThreads);
+  cfg.blockDim = dim3(512);
   cfg.dynamicSmemBytes = T::SMEM;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
