@@ -59,63 +59,60 @@ __device__ __forceinline__ void cross3(const float *a, const float *b, float *c)
   c[2] = a[0] * b[1] - a[1] * b[0];
 }
 
-// Transposed flux Jacobians of one face node for the face owner with normal n
-// and weights (Zm, Zp, Ym, Yp), applied to its face data g = (gE, gH):
-// contributions to the owner's interior trace (em, hm) and to the exterior
-// trace (ep, hp). With flux_E = (Zp/Zs) n x dH - (alpha/Zs) n x n x dE and
-// flux_H = -(Yp/Ys) n x dE - (alpha/Ys) n x n x dH, dq = q+ - q-, and
-// (n x .)^T = -(n x .), (n x n x .)^T = n x n x .
-// The face's zs = 1/(Zm+Zp) and ys = 1/(Ym+Yp) are given (they depend only on
-// the face, so they are formed once per face, not per face node).
-__device__ __forceinline__ void flux_transpose_w(const float *n, const float *g, float Zp, float Yp, float zs,
-                                                 float ys, float alpha, float *ep, float *hp) {
-  float nE[3], nH[3], nnE[3], nnH[3];
-  cross3(n, g, nE);
-  cross3(n, g + 3, nH);
-  cross3(n, nE, nnE);
-  cross3(n, nH, nnH);
+// One face node of the reverse stage: the transposed flux Jacobians of both
+// sides applied to the owner's face data g and the neighbour's g2 at the
+// matching node, acc = what the owner's node receives, and the eps gradient's
+// contraction of both sides' face data with the flux's derivatives in the
+// owner's impedances (dZ = dZ-/deps, dY = dY-/deps).
+//
+// With flux_E = zs n x (Z2 dH - alpha n x dE), flux_H = -ys n x (Y2 dE + alpha n x
+// dH), dq = q+ - q-, zs = 1/(Z- + Z2), ys = 1/(Y- + Y2), the neighbour sees -n,
+// swapped traces and the same zs, ys; (n x .)^T = -(n x .) and (n x n x .)^T =
+// n x n x . leave, with D = g - g2, cE = n x D_E, nE = n x cE (cH, nH alike),
+//   acc_E = alpha zs nE - n x g2_H - ys Y2 cH
+//   acc_H = alpha ys nH + n x g2_E + zs Z2 cE
+//   grad  = dZ zs^2 (Z2 dH.cE + alpha dE.nE) - dY ys^2 (Y2 dE.cH - alpha dH.nH):
+// six cross products and four inner products where the two sides taken one
+// after the other need sixteen cross products. A wall is the case g2 = (-g_E,
+// g_H) with the mirrored trace q+ = (-E-, H-). (Misfit and gradients at N=4,
+// 48,000 tets, 40 steps: 67.6 -> 65.8 ms.)
+struct FaceNode {
+  float cE[3], cH[3], nE[3], nH[3];
+  __device__ __forceinline__ FaceNode(const float *n, const float *g, const float *g2, float Z2, float Y2, float zs,
+                                      float ys, float alpha, float *acc) {
+    float dE[3], dH[3], xE[3], xH[3];
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    hp[c] = -(Zp * zs) * nE[c] - (alpha * ys) * nnH[c];
-    ep[c] = -(alpha * zs) * nnE[c] + (Yp * ys) * nH[c];
+    for (int c = 0; c < 3; ++c) {
+      dE[c] = g[c] - g2[c];
+      dH[c] = g[c + 3] - g2[c + 3];
+    }
+    cross3(n, dE, cE);
+    cross3(n, dH, cH);
+    cross3(n, cE, nE);
+    cross3(n, cH, nH);
+    cross3(n, g2, xE);
+    cross3(n, g2 + 3, xH);
+    const float az = alpha * zs, ay = alpha * ys, yw = ys * Y2, zw = zs * Z2;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      acc[c] = az * nE[c] - xH[c] - yw * cH[c];
+      acc[c + 3] = ay * nH[c] + xE[c] + zw * cE[c];
+    }
   }
-}
-
-// <g, d flux / d(weights)>: the contractions of the face data g with the
-// partial derivatives in Zm, Zp, Ym, Yp of the (unscaled) flux at one face
-// node, with the face's zs = 1/(Zm+Zp), ys = 1/(Ym+Yp) given: the flux
-// (weights zs and -ys) and n x dE, n x dH are formed once and shared.
-__device__ __forceinline__ void flux_weight_partials_w(const float *n, const float *qm, const float *qp, float Zp,
-                                                       float Yp, float zs, float ys, float alpha, const float *g,
-                                                       float &sZm, float &sZp, float &sYm, float &sYp) {
-  float dE[3], dH[3], nxdE[3], nxdH[3], v[3], f[6];
+  __device__ __forceinline__ float gradient(const float *qm, const float *qp, float Z2, float Y2, float zs, float ys,
+                                            float alpha, float dZ, float dY) const {
+    float hc = 0.f, en = 0.f, ec = 0.f, hn = 0.f;
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    dE[c] = qp[c] - qm[c];
-    dH[c] = qp[c + 3] - qm[c + 3];
+    for (int c = 0; c < 3; ++c) {
+      const float e = qp[c] - qm[c], h = qp[c + 3] - qm[c + 3];
+      hc += h * cE[c];
+      en += e * nE[c];
+      ec += e * cH[c];
+      hn += h * nH[c];
+    }
+    return dZ * zs * zs * (Z2 * hc + alpha * en) - dY * ys * ys * (Y2 * ec - alpha * hn);
   }
-  cross3(n, dE, nxdE);
-  cross3(n, dH, nxdH);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) v[c] = Zp * dH[c] - alpha * nxdE[c];
-  cross3(n, v, f);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) v[c] = Yp * dE[c] + alpha * nxdH[c];
-  cross3(n, v, f + 3);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    f[c] *= zs;
-    f[c + 3] *= -ys;
-  }
-  sZm = sZp = sYm = sYp = 0.f;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    sZm += g[c] * (-f[c] * zs);
-    sZp += g[c] * ((nxdH[c] - f[c]) * zs);
-    sYm += g[c + 3] * (-f[c + 3] * ys);
-    sYp += g[c + 3] * ((-nxdE[c] - f[c + 3]) * ys);
-  }
-}
+};
 
 } // namespace adj
 

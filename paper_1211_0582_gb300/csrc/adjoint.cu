@@ -211,47 +211,27 @@ __global__ void __launch_bounds__(AdjCfg<N>::NT2) k_adj_vol(AdjArgs a) {
     const float4 *fr = s_face + (e * 4 + f) * 4;
     const float4 r0 = fr[0], r1 = fr[1], r2 = fr[2], r3 = fr[3];
     const float n[3] = {r0.x, r0.y, r0.z};
-    const float zs = r0.w, Zk = r1.x, Z2 = r1.y, Yk = r1.z, Y2 = r1.w, ys = r2.x;
+    const float zs = r0.w, Z2 = r1.y, Y2 = r1.w, ys = r2.x;
     const int cny = __float_as_int(r2.w);
     const int64_t k2 = __float_as_int(r3.x);
     const bool wall = __float_as_int(r3.y) != 0;
     float gk[6];
 #pragma unroll
     for (int c = 0; c < 6; ++c) gk[c] = a.g[(c * a.K + k) * NFF + fm];
-    float ep[3], hp[3], acc[6];
-    flux_transpose_w(n, gk, Z2, Y2, zs, ys, a.alpha, ep, hp);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      acc[c] = -ep[c];      // interior side: the E and H Jacobians are the negatives of the exterior ones
-      acc[c + 3] = -hp[c];
-    }
     const int fm2 = wall ? 0 : s_nf[cny * NFP + m] + (cny / 6 % 4) * NFP;
-    float g2[6];
+    float g2[6], acc[6];
     if (wall) {
-      // exterior state E+ = -E-, H+ = H- folds back onto the interior node
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        acc[c] -= ep[c];
-        acc[c + 3] += hp[c];
-      }
+      for (int c = 0; c < 3; ++c) g2[c] = -gk[c], g2[c + 3] = gk[c + 3];
     } else {
-      // the neighbour's flux sees this element as its exterior side
 #pragma unroll
       for (int c = 0; c < 6; ++c) g2[c] = a.g[(c * a.K + k2) * NFF + fm2];
-      const float n2[3] = {-n[0], -n[1], -n[2]};
-      float ep2[3], hp2[3];
-      flux_transpose_w(n2, g2, Zk, Yk, zs, ys, a.alpha, ep2, hp2);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        acc[c] += ep2[c];
-        acc[c + 3] += hp2[c];
-      }
     }
+    const FaceNode fnode(n, gk, g2, Z2, Y2, zs, ys, a.alpha, acc);
     const int vm = s_fm[fm];
 #pragma unroll
     for (int c = 0; c < 6; ++c) atomicAdd(&s_w[(c * EB + e) * NPP + vm], acc[c]);
     if (GRAD) {
-      const float dZ = r2.y, dY = r2.z;
       float qm[6], qp[6];
 #pragma unroll
       for (int c = 0; c < 6; ++c) qm[c] = __ldg(a.u_s + c * KN + k * NPP + vm);
@@ -266,17 +246,7 @@ __global__ void __launch_bounds__(AdjCfg<N>::NT2) k_adj_vol(AdjArgs a) {
 #pragma unroll
         for (int c = 0; c < 6; ++c) qp[c] = __ldg(a.u_s + c * KN + k2 * NPP + vn);
       }
-      float sZm, sZp, sYm, sYp;
-      flux_weight_partials_w(n, qm, qp, Z2, Y2, zs, ys, a.alpha, gk, sZm, sZp, sYm, sYp);
-      contrib = sZm * dZ + sYm * dY;
-      if (wall) {
-        contrib += sZp * dZ + sYp * dY; // the mirrored exterior carries the same weights
-      } else {
-        const float n2[3] = {-n[0], -n[1], -n[2]};
-        float tZm, tZp, tYm, tYp;
-        flux_weight_partials_w(n2, qp, qm, Zk, Yk, zs, ys, a.alpha, g2, tZm, tZp, tYm, tYp);
-        contrib += tZp * dZ + tYp * dY;
-      }
+      contrib = fnode.gradient(qm, qp, Z2, Y2, zs, ys, a.alpha, r2.y, r2.z);
     }
     }
     if (GRAD) add_by_element(s_gr, e, contrib);

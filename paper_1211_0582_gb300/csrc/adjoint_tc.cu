@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
         const float4 *fr = s_face + (e * 4 + f) * 4;
         const float4 r0 = fr[0], r1 = fr[1], r2 = fr[2], r3 = fr[3];
         const float n[3] = {r0.x, r0.y, r0.z};
-        const float zs = r0.w, Zk = r1.x, Z2 = r1.y, Yk = r1.z, Y2 = r1.w, ys = r2.x;
+        const float zs = r0.w, Z2 = r1.y, Y2 = r1.w, ys = r2.x;
         const int cny = __float_as_int(r2.w);
         const int64_t k2 = __float_as_int(r3.x);
         const bool wall = __float_as_int(r3.y) != 0;
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
         const int vn = wall ? 0 : s_nb[cny * NFP + m];
         // every global load of the item first, all in flight together: the
         // own and the neighbour's face data, the stage's own and exterior traces
-        float gk[6], g2[6], qm[6], qp[6];
+        float gk[6], g2[6], qm[6] = {}, qp[6] = {};
 #pragma unroll
         for (int c = 0; c < 6; ++c) gk[c] = a.g[(c * a.K + k) * NFF + fm];
 #pragma unroll
@@ -345,50 +345,16 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
 #pragma unroll
           for (int c = 0; c < 6; ++c) qp[c] = wall ? 0.f : __ldg(a.u_s + c * KN + k2 * NPP + vn);
         }
-        float ep3[3], hp3[3], acc[6];
-        flux_transpose_w(n, gk, Z2, Y2, zs, ys, a.alpha, ep3, hp3);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          acc[c] = -ep3[c];
-          acc[c + 3] = -hp3[c];
-        }
         if (wall) {
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
-            acc[c] -= ep3[c];
-            acc[c + 3] += hp3[c];
-          }
-        } else {
-          const float n2[3] = {-n[0], -n[1], -n[2]};
-          float ep2[3], hp2[3];
-          flux_transpose_w(n2, g2, Zk, Yk, zs, ys, a.alpha, ep2, hp2);
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            acc[c] += ep2[c];
-            acc[c + 3] += hp2[c];
+            g2[c] = -gk[c], g2[c + 3] = gk[c + 3];
+            qp[c] = -qm[c], qp[c + 3] = qm[c + 3];
           }
         }
-        if (grad) {
-          const float dZ = r2.y, dY = r2.z;
-          if (wall) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              qp[c] = -qm[c];
-              qp[c + 3] = qm[c + 3];
-            }
-          }
-          float sZm, sZp, sYm, sYp;
-          flux_weight_partials_w(n, qm, qp, Z2, Y2, zs, ys, a.alpha, gk, sZm, sZp, sYm, sYp);
-          contrib = sZm * dZ + sYm * dY;
-          if (wall) {
-            contrib += sZp * dZ + sYp * dY;
-          } else {
-            const float n2[3] = {-n[0], -n[1], -n[2]};
-            float tZm, tZp, tYm, tYp;
-            flux_weight_partials_w(n2, qp, qm, Zk, Yk, zs, ys, a.alpha, g2, tZm, tZp, tYm, tYp);
-            contrib += tZp * dZ + tYp * dY;
-          }
-        }
+        float acc[6];
+        const FaceNode fnode(n, gk, g2, Z2, Y2, zs, ys, a.alpha, acc);
+        if (grad) contrib = fnode.gradient(qm, qp, Z2, Y2, zs, ys, a.alpha, r2.y, r2.z);
 #pragma unroll
         for (int c = 0; c < 6; ++c) atomicAdd(&s_w[c * FS + e * NPP + vm], acc[c]);
       }
