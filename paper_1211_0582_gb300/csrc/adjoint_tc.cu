@@ -45,6 +45,7 @@
 #include "adj_common.cuh"
 #include "flux.cuh"
 #include "tc_common.cuh"
+#include "tiles.cuh"
 #include "umma.cuh"
 
 namespace dgmx {
@@ -127,7 +128,7 @@ __device__ uint32_t g_adj_trace[kAdjTraceBlocks * kAdjTraceTiles * kAdjEvents];
 
 template <int N>
 __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
-    k_adj_tc(AdjArgs a, const uint4 *__restrict__ ops, int ntiles, long long wait_limit, int *err_flag) {
+    k_adj_tc(AdjArgs a, const uint4 *__restrict__ ops, TileMap<AT<N>::TE> tm, long long wait_limit, int *err_flag) {
   using T = AT<N>;
   constexpr int NP = T::NP, NPP = T::NPP, NFP = T::NFP, NFF = T::NFF, FS = T::FS, NT = T::NT, NB = T::NB;
   constexpr int K1 = T::K1, CPP = T::CPP, NCH = T::NCH, GPP = T::GPP, GCH = T::GCH;
@@ -204,8 +205,8 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
   // barS, face and element data on barF; the next tile's rows are requested as
   // soon as the epilogue has read this tile's, its face data at the tile's end
   auto stage_rows = [&](int t) {
-    const int64_t kb = int64_t(t) * T::TE;
-    const uint32_t nb = uint32_t(a.K - kb < T::TE ? a.K - kb : T::TE), bytes = nb * NPP * 4u;
+    const int64_t kb = tm.start(t);
+    const uint32_t nb = uint32_t(tm.size(t, a.K)), bytes = nb * NPP * 4u;
     umma::mbar_arrive_expect_tx(barS, (grad ? 15u : 12u) * bytes);
     for (int f = 0; f < 6; ++f) {
       umma::bulk_g2s(s_lr + f * FS, a.lr_in + f * KN + kb * NPP, bytes, barS);
@@ -215,14 +216,14 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
       for (int f = 0; f < 3; ++f) umma::bulk_g2s(s_rs + f * FS, a.rhs_s + f * KN + kb * NPP, bytes, barS);
   };
   auto stage_faces = [&](int t) {
-    const int64_t kb = int64_t(t) * T::TE;
-    const uint32_t nb = uint32_t(a.K - kb < T::TE ? a.K - kb : T::TE);
+    const int64_t kb = tm.start(t);
+    const uint32_t nb = uint32_t(tm.size(t, a.K));
     umma::mbar_arrive_expect_tx(barF, nb * (64u + G_STRIDE * 4u + 256u));
     umma::bulk_g2s(smem + T::OFF_FG, a.fgeo + kb * 4, nb * 64u, barF);
     umma::bulk_g2s(smem + T::OFF_GEO, a.geo + kb * G_STRIDE, nb * G_STRIDE * 4u, barF);
     umma::bulk_g2s(s_face, a.fcon + kb * 16, nb * 256u, barF);
   };
-  if (tid == 0 && int(blockIdx.x) < ntiles) {
+  if (tid == 0 && int(blockIdx.x) < tm.ntiles) {
     stage_rows(blockIdx.x);
     stage_faces(blockIdx.x);
   }
@@ -232,17 +233,17 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
 #ifdef DGMX_STAGE_TIMING
   const long long at_t0 = clock64();
 #endif
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+  for (int tile = blockIdx.x; tile < tm.ntiles; tile += gridDim.x) {
 #ifdef DGMX_STAGE_TIMING
     const int itn = (tile - int(blockIdx.x)) / int(gridDim.x);
 #endif
     AT_MARK(0);
-    if (tile + int(gridDim.x) >= ntiles) pdl_launch_next(); // this block's last tile
-    const int64_t k0 = int64_t(tile) * T::TE;
-    const int ne = int(a.K - k0 < T::TE ? a.K - k0 : T::TE);
+    if (tile + int(gridDim.x) >= tm.ntiles) pdl_launch_next(); // this block's last tile
+    const int64_t k0 = tm.start(tile);
+    const int ne = tm.size(tile, a.K);
     const bool live = lane_used && e_loc < ne;
 
-    const bool more = tile + int(gridDim.x) < ntiles;
+    const bool more = tile + int(gridDim.x) < tm.ntiles;
     // ---- A. the tile's lambda_r, lambda_u, face and element data (bulk copies
     // requested during the previous tile)
     const bool okS = umma::mbar_wait_bounded(barS, phase, wlim) && umma::mbar_wait_bounded(barF, phase, wlim);
@@ -619,11 +620,11 @@ cudaError_t launch_adj_tc_order(const AdjArgs &a, const AdjTcState &st, long lon
   const int tmem_fit = 512 / T::TCOLS;
   if (per_sm > tmem_fit) per_sm = tmem_fit;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const int ntiles = int((a.K + T::TE - 1) / T::TE);
   const int cap = per_sm * st.sms;
-  const int grid = ntiles < cap ? ntiles : cap;
+  const TileMap<T::TE> tm = make_tiles<T::TE>(a.K, cap);
+  const int grid = tm.ntiles < cap ? tm.ntiles : cap;
   return launch_pdl(kern, dim3(unsigned(grid)), dim3(T::NT), size_t(T::SMEM), s, a,
-                    reinterpret_cast<const uint4 *>(st.d_ops), ntiles, wait_limit, flag);
+                    reinterpret_cast<const uint4 *>(st.d_ops), tm, wait_limit, flag);
 }
 
 } // namespace

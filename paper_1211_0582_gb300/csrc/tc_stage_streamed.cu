@@ -34,6 +34,7 @@
 #include "../../include/dgmx.h"
 #include "flux.cuh"
 #include "tc_common.cuh"
+#include "tiles.cuh"
 #include "umma.cuh"
 
 namespace dgmx {
@@ -112,7 +113,7 @@ __host__ __device__ constexpr uint32_t slice_offset(int st) {
 
 template <int N, int MODE, bool BF16>
 __global__ void __launch_bounds__(kThreadsS, 1)
-    k_stage_tc_streamed(StageArgs a, const uint8_t *__restrict__ stream, int ntiles, int *err_flag) {
+    k_stage_tc_streamed(StageArgs a, const uint8_t *__restrict__ stream, TileMap<kTileS> tm, int *err_flag) {
   using T = TS<N>;
   constexpr int NP = T::NP, NFP = T::NFP, NPP = T::NPP, NFF = T::NFF, FS = T::FS, NB = T::NB;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -197,7 +198,7 @@ __global__ void __launch_bounds__(kThreadsS, 1)
     ++jstep;
     return stream_ok;
   };
-  if (issuer && int(blockIdx.x) < ntiles)
+  if (issuer && int(blockIdx.x) < tm.ntiles)
     for (int j = 0; j < kSlots; ++j) produce(uint32_t(j));
 
   // field split (all 16 warps): warp w owns operand rows 8w..8w+7 (lane ->
@@ -243,29 +244,29 @@ __global__ void __launch_bounds__(kThreadsS, 1)
 
   // warm L2 with the fields of the CTA's next tile and the residual of this one
   auto prefetch = [&](int tu, int tr) {
-    if (tu < ntiles) {
-      const int64_t kb = int64_t(tu) * kTileS, nb = a.K - kb < kTileS ? a.K - kb : kTileS;
+    if (tu < tm.ntiles) {
+      const int64_t kb = tm.start(tu), nb = tm.size(tu, a.K);
       for (int f = 0; f < 6; ++f) umma::prefetch_l2(a.u + f * KN + kb * NPP, uint32_t(nb * NPP * 4));
       umma::prefetch_l2(a.fconn + kb * 4, uint32_t(nb * 32));
       umma::prefetch_l2(a.fgeo + kb * 4, uint32_t(nb * 64));
       umma::prefetch_l2(a.fmat + kb * 4, uint32_t(nb * 64));
     }
-    if (MODE == MODE_LSERK && a.rk_a != 0.f && tr < ntiles) {
-      const int64_t kb = int64_t(tr) * kTileS, nb = a.K - kb < kTileS ? a.K - kb : kTileS;
+    if (MODE == MODE_LSERK && a.rk_a != 0.f && tr >= 0) {
+      const int64_t kb = tm.start(tr), nb = tm.size(tr, a.K);
       for (int f = 0; f < 6; ++f) umma::prefetch_l2(a.res + f * KN + kb * NPP, uint32_t(nb * NPP * 4));
     }
   };
-  if (tid == 32 && int(blockIdx.x) < ntiles) prefetch(blockIdx.x, -1);
+  if (tid == 32 && int(blockIdx.x) < tm.ntiles) prefetch(blockIdx.x, -1);
 
   uint32_t phase = 0;
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+  for (int tile = blockIdx.x; tile < tm.ntiles; tile += gridDim.x) {
 #ifdef DGMX_STAGE_TIMING
     const int itn = (tile - int(blockIdx.x)) / int(gridDim.x);
 #endif
     TS_MARK(tid == 0, 0);
-    if (tile + int(gridDim.x) >= ntiles) pdl_launch_next(); // this block's last tile
-    const int64_t k0 = int64_t(tile) * kTileS;
-    const int ne = int(a.K - k0 < kTileS ? a.K - k0 : kTileS);
+    if (tile + int(gridDim.x) >= tm.ntiles) pdl_launch_next(); // this block's last tile
+    const int64_t k0 = tm.start(tile);
+    const int ne = tm.size(tile, a.K);
     bool ok = true;
     if (tid == 32) prefetch(tile + int(gridDim.x), tile);
 
@@ -720,10 +721,10 @@ cudaError_t launch_streamed_kernel(const StageArgs &a, const TcState &st, int *f
   auto kern = k_stage_tc_streamed<N, MODE, BF16>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM);
   if (e != cudaSuccess) return e;
-  const int ntiles = int((a.K + kTileS - 1) / kTileS);
-  const int grid = ntiles < st.sms ? ntiles : st.sms;
+  const TileMap<kTileS> tm = make_tiles<kTileS>(a.K, st.sms);
+  const int grid = tm.ntiles < st.sms ? tm.ntiles : st.sms;
   return launch_pdl(kern, dim3(unsigned(grid)), dim3(kThreadsS), size_t(T::SMEM), s, a,
-                    static_cast<const uint8_t *>(st.d_ops), ntiles, flag);
+                    static_cast<const uint8_t *>(st.d_ops), tm, flag);
 }
 
 template <int N>
