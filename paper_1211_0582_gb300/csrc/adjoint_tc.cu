@@ -94,14 +94,23 @@ struct AT {
   static constexpr int TB = rup(6 * FS * 4, 128);
   static constexpr int OFF_LR = rup(OPS, 128); // fp32 [6][FS] lambda_r of the tile
   static constexpr int OFF_LU = OFF_LR + TB;   // fp32 [6][FS] lambda_u of the tile
-  static constexpr int OFF_W = OFF_LU + TB;    // fp32 [6][FS] transposed-flux contributions
-  static constexpr int OFF_RS = OFF_W + TB;    // fp32 [3][FS] E rows of the stage's right-hand side
-  static constexpr int OFF_FACE = OFF_RS + rup(3 * FS * 4, 128); // float4 [80][4] per-face constants
+  // what each face node contributes to its volume node, fp32 [NFF][RSX] with the
+  // six fields of an element together (an odd row stride in units of 8 bytes:
+  // the face loop's stores hit different banks); the same bytes hold the E rows
+  // of the stage's right-hand side, fp32 [3][FS], until the face loop. (Floating
+  // point atomics on the volume nodes in shared memory took the face loop 22.8k
+  // cycles per tile at N = 4 and the epilogue 5.0k; stored per face node and
+  // gathered by the epilogue 15.7k and 7.0k.)
+  static constexpr int RSX = TE * 6 % 4 == 2 ? TE * 6 : TE * 6 + 2;
+  static constexpr int XB = NFF * RSX > 3 * FS ? NFF * RSX * 4 : 3 * FS * 4;
+  static constexpr int OFF_X = OFF_LU + TB, OFF_RS = OFF_X;
+  static constexpr int OFF_FACE = OFF_X + rup(XB, 128); // float4 [80][4] per-face constants
   static constexpr int OFF_FG = OFF_FACE + kAdjTile * 4 * 64; // float4 [80] {n, Fscale}
   static constexpr int OFF_GEO = OFF_FG + kAdjTile * 4 * 16;  // float [20][G_STRIDE]
   static constexpr int OFF_TAB = OFF_GEO + kAdjTile * G_STRIDE * 4;
   // u32 [128] row maxima, float [128] inverse row scales, float [20] gradient partials
-  static constexpr int OFF_MX = OFF_TAB + rup(NFF + 2 * kConnKinds * NFP, 16);
+  static constexpr int OFF_N2F = OFF_TAB + rup(NFF + 2 * kConnKinds * NFP, 16); // u32 [NP] face nodes of each node
+  static constexpr int OFF_MX = OFF_N2F + rup(NP * 4, 16);
   static constexpr int OFF_BAR = OFF_MX + 2 * 128 * 4 + rup(kAdjTile, 4) * 4; // barS, barF, barD, barL; TMEM slot
   static constexpr int SMEM = OFF_BAR + 48;
   static_assert(SMEM <= 232448, "the reverse tile does not fit in shared memory");
@@ -135,13 +144,14 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
   extern __shared__ __align__(1024) uint8_t smem[];
   float *s_lr = reinterpret_cast<float *>(smem + T::OFF_LR);
   float *s_lu = reinterpret_cast<float *>(smem + T::OFF_LU);
-  float *s_w = reinterpret_cast<float *>(smem + T::OFF_W);
+  float *s_x = reinterpret_cast<float *>(smem + T::OFF_X);
   float *s_rs = reinterpret_cast<float *>(smem + T::OFF_RS);
   float4 *s_face = reinterpret_cast<float4 *>(smem + T::OFF_FACE);
   const float4 *s_fg = reinterpret_cast<const float4 *>(smem + T::OFF_FG);
   const float *s_geo = reinterpret_cast<const float *>(smem + T::OFF_GEO);
   uint8_t *s_fm = smem + T::OFF_TAB;
   uint8_t *s_nb = s_fm + NFF, *s_nf = s_nb + kConnKinds * NFP;
+  uint32_t *s_n2f = reinterpret_cast<uint32_t *>(smem + T::OFF_N2F); // up to three face nodes, a byte each, 255: none
   uint32_t *s_rmx = reinterpret_cast<uint32_t *>(smem + T::OFF_MX); // row maxima (float bits)
   float *s_inv = reinterpret_cast<float *>(s_rmx + 128);            // inverse row scales (compact rows)
   float *s_gr = s_inv + 128;                                         // eps-gradient partial per element
@@ -161,7 +171,13 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
   for (int i = tid; i < T::OPS / 16; i += NT) reinterpret_cast<uint4 *>(smem)[i] = __ldg(ops + i);
   for (int i = tid; i < NFF + 2 * kConnKinds * NFP; i += NT)
     s_fm[i] = i < NFF ? a.fmask[i] : i < NFF + kConnKinds * NFP ? a.nbrtab[i - NFF] : a.nbrface[i - NFF - kConnKinds * NFP];
-  for (int i = tid; i < 6 * FS; i += NT) s_w[i] = 0.f;
+  for (int i = tid; i < NP; i += NT) {
+    uint32_t w = 0u;
+    int shift = 0;
+    for (int fm = 0; fm < NFF; ++fm)
+      if (a.fmask[fm] == i) w |= uint32_t(fm) << shift, shift += 8;
+    s_n2f[i] = shift < 24 ? w | (0xffffffffu << shift) : w | 0xff000000u;
+  }
   for (int i = tid; i < 128; i += NT) s_rmx[i] = 0u, s_inv[i] = 1.f;
   for (int i = tid; i < kAdjTile; i += NT) s_gr[i] = 0.f;
   if (tid == 0) {
@@ -315,7 +331,7 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
 
     // ---- D. transposed flux Jacobians (interior side with the element's own
     // g, exterior side with the neighbour's g at the matching face node) into
-    // s_w, and the impedance-weight terms of the gradient; one face node per
+    // s_x, and the impedance-weight terms of the gradient; one face node per
     // item, whole rounds (every lane takes part in the per-element sums)
     for (int it0 = 0; it0 < ne * NFF; it0 += NT) {
       const int it = it0 + tid;
@@ -356,8 +372,10 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
         float acc[6];
         const FaceNode fnode(n, gk, g2, Z2, Y2, zs, ys, a.alpha, acc);
         if (grad) contrib = fnode.gradient(qm, qp, Z2, Y2, zs, ys, a.alpha, r2.y, r2.z);
-#pragma unroll
-        for (int c = 0; c < 6; ++c) atomicAdd(&s_w[c * FS + e * NPP + vm], acc[c]);
+        float2 *x = reinterpret_cast<float2 *>(s_x + fm * T::RSX + e * 6);
+        x[0] = make_float2(acc[0], acc[1]);
+        x[1] = make_float2(acc[2], acc[3]);
+        x[2] = make_float2(acc[4], acc[5]);
       }
       if (grad) add_by_element(s_gr, e, contrib);
     }
@@ -423,12 +441,18 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
         for (int h = 0; h < 2; ++h) {
           const int i = i0 + 4 * h;
           if (i < NPP) {
-            const float4 sw4 = *reinterpret_cast<const float4 *>(s_w + soff + i);
-            // read once: cleared here for the next tile (entries no live row reads are never written)
-            *reinterpret_cast<float4 *>(s_w + soff + i) = make_float4(0.f, 0.f, 0.f, 0.f);
+            float swv[4]; // the node's face-node contributions (up to three faces meet at a node)
+#pragma unroll
+            for (int n = 0; n < 4; ++n) {
+              swv[n] = 0.f;
+              uint32_t w = i + n < NP ? s_n2f[i + n] : 0xffffffffu;
+#pragma unroll
+              for (int j = 0; j < 3; ++j, w >>= 8)
+                if ((w & 0xffu) != 0xffu) swv[n] += s_x[(w & 0xffu) * T::RSX + ridx];
+            }
             const float4 lu4 = *reinterpret_cast<const float4 *>(s_lu + soff + i);
             const float4 lr4 = *reinterpret_cast<const float4 *>(s_lr + soff + i);
-            const float swv[4] = {sw4.x, sw4.y, sw4.z, sw4.w}, luv[4] = {lu4.x, lu4.y, lu4.z, lu4.w},
+            const float luv[4] = {lu4.x, lu4.y, lu4.z, lu4.w},
                         lrv[4] = {lr4.x, lr4.y, lr4.z, lr4.w};
             float o[4], p[4];
 #pragma unroll
