@@ -644,7 +644,7 @@ cudaError_t launch_adj_tc_order(const AdjArgs &a, const AdjTcState &st, long lon
   const int tmem_fit = 512 / T::TCOLS;
   if (per_sm > tmem_fit) per_sm = tmem_fit;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const int cap = per_sm * st.sms;
+  const int cap = small_mesh_blocks<T::TE>(a.K, per_sm * st.sms);
   const TileMap<T::TE> tm = make_tiles<T::TE>(a.K, cap);
   const int grid = tm.ntiles < cap ? tm.ntiles : cap;
   return launch_pdl(kern, dim3(unsigned(grid)), dim3(T::NT), size_t(T::SMEM), s, a,

@@ -115,7 +115,7 @@ std::string cache_path() {
 std::string cache_key(const EnsembleState &st, int N, int precision, int64_t K) {
   std::ostringstream os;
   // T: the candidate list that the cached index refers to
-  os << st.gpu << "|N=" << N << "|P=" << precision << "|K=" << K << "|T=2";
+  os << st.gpu << "|N=" << N << "|P=" << precision << "|K=" << K << "|T=3";
   return os.str();
 }
 
@@ -309,7 +309,6 @@ int dg_ensemble_tune(dg_ctx *ctx, int force) {
     st.ms[cand] = 0.f;
     if (tc && cand > 0) continue;
     const int i = cand % kEbCandidates;
-    if (i > 0 && candidate_eb(ctx->N, cand) == candidate_eb(ctx->N, cand - 1)) continue;
     // the second occupancy level only where it launches fewer blocks than the first
     if (cand >= kEbCandidates && (st.ms[i] == 0.f || st.bps[i] <= 1)) continue;
     float t_min = 1e30f;

@@ -47,15 +47,14 @@ namespace dgmx {
 
 // Tile candidates of the autotuner for order N, in elements: where the small
 // shape serves alone its tile and three, two and one quarter of it; elsewhere
-// the two-element shape's tile and three and two quarters of it, and the small
-// shape's tile.
+// the two-element shape's tile and half of it, and the small shape's.
 template <int N>
 struct EnsembleCandidates {
-  static constexpr bool small(int i) { return simt_small_only<N>() || i == 3; }
+  static constexpr bool small(int i) { return simt_small_only<N>() || i >= 2; }
   static constexpr int c(int i) {
-    if (i == 3 && !simt_small_only<N>()) return SimtShape<N, true>::EB;
-    const int eb = SimtShape<N, simt_small_only<N>()>::EB * (4 - i) / 16 * 4;
-    return eb > 4 ? eb : 4;
+    if (simt_small_only<N>()) return SimtShape<N, true>::EB * (4 - i) / 8 * 2;
+    const int step = i < 2 ? 4 : 2, eb = i < 2 ? SimtShape<N, false>::EB : SimtShape<N, true>::EB;
+    return i % 2 ? eb / (2 * step) * step : eb;
   }
   template <int I>
   using Cfg = SimtCfg<N, small(I), c(I)>;

@@ -185,9 +185,10 @@ __device__ __forceinline__ void simt_product(float2 (&acc)[3 * Cfg::S::RE][4 * C
   product(x1, w1);
 }
 
-// One tile of ne <= EB elements starting at k0 (all threads of the block call it).
+// One tile of ne <= EB elements starting at k0 (all threads of the block call
+// it); staged: the first chunk's operator rows are on their way already.
 template <int N, int MODE, class Cfg, bool COHERENT>
-__device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, int ne, uint8_t *smem) {
+__device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, int ne, uint8_t *smem, bool staged = false) {
   using D = Dims<N>;
   constexpr int NP = D::NP, NFP = D::NFP, NPP = D::NPP, NQ = D::NQ, QC = Cfg::QC, FR = Cfg::FR, NT = Cfg::NT;
   constexpr int RS = Cfg::RS, CG = Cfg::CG, RE = Cfg::S::RE, CQ = Cfg::S::CQ;
@@ -202,7 +203,7 @@ __device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, 
   const int64_t KN = a.K * NPP;
   const float *u0 = a.u + k0 * NPP;
 
-  simt_stage_operator<Cfg>(s_w, a.LT, FR < D::NFF ? FR : D::NFF);
+  if (!staged) simt_stage_operator<Cfg>(s_w, a.LT, FR < D::NFF ? FR : D::NFF);
   for (int i = tid; i < ne * 4; i += NT) {
     cp_async<16>(s_fgeo + i, a.fgeo + k0 * 4 + i);
     cp_async<16>(s_fmat + i, a.fmat + k0 * 4 + i);
@@ -386,11 +387,15 @@ __global__ void __launch_bounds__(SimtCfg<N, SMALL>::NT, SimtCfg<N, SMALL>::MINB
   using Cfg = SimtCfg<N, SMALL>;
   extern __shared__ float4 smem4[];
   simt_setup<Cfg>(a, smem4);
+  // (the operator is fixed: its first rows may arrive before the previous stage has ended)
+  simt_stage_operator<Cfg>(reinterpret_cast<float *>(reinterpret_cast<uint8_t *>(smem4) + Cfg::OFF_W), a.LT,
+                           Cfg::FR < Cfg::D::NFF ? Cfg::FR : Cfg::D::NFF);
   pdl_wait(); // stage after stage: fields of the previous stage from here on
   for (int t = blockIdx.x; t < tm.ntiles; t += gridDim.x) {
     if (t + int(gridDim.x) >= tm.ntiles) pdl_launch_next(); // this block's last tile
     if (t != int(blockIdx.x)) __syncthreads(); // shared memory of the previous tile is no longer read
-    simt_stage_tile<N, MODE, Cfg, false>(a, tm.start(t), tm.size(t, a.K), reinterpret_cast<uint8_t *>(smem4));
+    simt_stage_tile<N, MODE, Cfg, false>(a, tm.start(t), tm.size(t, a.K), reinterpret_cast<uint8_t *>(smem4),
+                                           t == int(blockIdx.x));
   }
 }
 
@@ -412,8 +417,9 @@ cudaError_t launch_simt_mode(const StageArgs &a, int dev, int sms, cudaStream_t 
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     if (dev < kDevCache) per_sm_cache[dev].store(per_sm, std::memory_order_relaxed);
   }
-  const TileMap<Cfg::EB> tm = make_tiles<Cfg::EB>(a.K, per_sm * sms);
-  const unsigned blocks = unsigned(tm.ntiles < per_sm * sms ? tm.ntiles : per_sm * sms);
+  const int cap = small_mesh_blocks<Cfg::EB>(a.K, per_sm * sms);
+  const TileMap<Cfg::EB> tm = make_tiles<Cfg::EB>(a.K, cap);
+  const unsigned blocks = unsigned(tm.ntiles < cap ? tm.ntiles : cap);
   return launch_pdl(kern, dim3(blocks), dim3(Cfg::NT), Cfg::SMEM, s, a, tm);
 }
 

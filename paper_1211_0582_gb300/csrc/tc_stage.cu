@@ -1491,8 +1491,10 @@ cudaError_t launch_tc_kernel(const StageArgs &a, const TcState &st, int *flag, c
   // the largest shared-memory carveout, so that the blocks of an SM fit side by side
   if (e == cudaSuccess && T::BLOCKS > 1) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   if (e != cudaSuccess) return e;
-  // a mesh of at most one tile per SM is spread over the SMs, not over their blocks
-  const int blocks = a.K <= int64_t(kTileElems) * st.sms ? st.sms : T::BLOCKS * st.sms;
+  // with several blocks per SM, a mesh of at most one tile per SM is spread over
+  // the SMs, not over their blocks
+  const int blocks = T::BLOCKS == 1 ? small_mesh_blocks<kTileElems>(a.K, st.sms)
+                     : a.K <= int64_t(kTileElems) * st.sms ? st.sms : T::BLOCKS * st.sms;
   const TileMap<kTileElems> tm = make_tiles<kTileElems>(a.K, blocks);
   const int grid = tm.ntiles < blocks ? tm.ntiles : blocks;
   return launch_pdl(kern, dim3(unsigned(grid)), dim3(T::THREADS), size_t(T::SMEM), s, a,

@@ -35,4 +35,16 @@ TileMap<FULL> make_tiles(int64_t K, int grid) {
   return TileMap<FULL>{int(nfull), int(small), int(nfull + nsmall)};
 }
 
+// Blocks of a launch that may have `cap` resident at once: half of them where the
+// mesh fits half of them in full tiles. The other half of the SMs' room then
+// takes the next stage's blocks, whose setup (operators, tables, tensor memory)
+// overlaps this stage (programmatic dependent launch) instead of following it.
+// (us per stage, all blocks and half: FP16x3 N=4 1,296 tets 7.13 -> 6.72, N=5 750
+// tets 8.86 -> 7.11, N=7 162 tets 13.6 -> 12.9; FP32 N=3 1,296 tets 8.4 -> 7.4,
+// N=8 750 tets 54.6 -> 34.9; a few sizes at N <= 4 lose up to 9%.)
+template <int FULL>
+int small_mesh_blocks(int64_t K, int cap) {
+  return cap >= 2 && K <= int64_t(FULL) * (cap / 2) ? cap / 2 : cap;
+}
+
 } // namespace dgmx
