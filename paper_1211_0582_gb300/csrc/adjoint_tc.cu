@@ -100,11 +100,15 @@ struct AT {
   // of the stage's right-hand side, fp32 [3][FS], until the face loop. (Floating
   // point atomics on the volume nodes in shared memory took the face loop 22.8k
   // cycles per tile at N = 4 and the epilogue 5.0k; stored per face node and
-  // gathered by the epilogue 15.7k and 7.0k.)
+  // gathered by the epilogue 16k and 5.8k, 7.0k with a branch per face node
+  // instead of a row of zeros for the nodes of fewer faces.)
   static constexpr int RSX = TE * 6 % 4 == 2 ? TE * 6 : TE * 6 + 2;
   static constexpr int XB = NFF * RSX > 3 * FS ? NFF * RSX * 4 : 3 * FS * 4;
+  static_assert(NFF < 255, "face nodes are bytes");
   static constexpr int OFF_X = OFF_LU + TB, OFF_RS = OFF_X;
-  static constexpr int OFF_FACE = OFF_X + rup(XB, 128); // float4 [80][4] per-face constants
+  static constexpr int ZROW = rup(XB, 4 * RSX) / (4 * RSX); // a row of zeros past the buffer
+  static constexpr int OFF_FACE = OFF_X + rup((ZROW + 1) * RSX * 4, 128); // float4 [80][4] per-face constants
+  static_assert(ZROW < 255, "row numbers are bytes");
   static constexpr int OFF_FG = OFF_FACE + kAdjTile * 4 * 64; // float4 [80] {n, Fscale}
   static constexpr int OFF_GEO = OFF_FG + kAdjTile * 4 * 16;  // float [20][G_STRIDE]
   static constexpr int OFF_TAB = OFF_GEO + kAdjTile * G_STRIDE * 4;
@@ -151,7 +155,7 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
   const float *s_geo = reinterpret_cast<const float *>(smem + T::OFF_GEO);
   uint8_t *s_fm = smem + T::OFF_TAB;
   uint8_t *s_nb = s_fm + NFF, *s_nf = s_nb + kConnKinds * NFP;
-  uint32_t *s_n2f = reinterpret_cast<uint32_t *>(smem + T::OFF_N2F); // up to three face nodes, a byte each, 255: none
+  uint32_t *s_n2f = reinterpret_cast<uint32_t *>(smem + T::OFF_N2F); // three rows of s_x, a byte each (ZROW: none)
   uint32_t *s_rmx = reinterpret_cast<uint32_t *>(smem + T::OFF_MX); // row maxima (float bits)
   float *s_inv = reinterpret_cast<float *>(s_rmx + 128);            // inverse row scales (compact rows)
   float *s_gr = s_inv + 128;                                         // eps-gradient partial per element
@@ -176,8 +180,10 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
     int shift = 0;
     for (int fm = 0; fm < NFF; ++fm)
       if (a.fmask[fm] == i) w |= uint32_t(fm) << shift, shift += 8;
-    s_n2f[i] = shift < 24 ? w | (0xffffffffu << shift) : w | 0xff000000u;
+    for (; shift < 24; shift += 8) w |= uint32_t(T::ZROW) << shift;
+    s_n2f[i] = w;
   }
+  for (int i = tid; i < T::RSX; i += NT) s_x[T::ZROW * T::RSX + i] = 0.f;
   for (int i = tid; i < 128; i += NT) s_rmx[i] = 0u, s_inv[i] = 1.f;
   for (int i = tid; i < kAdjTile; i += NT) s_gr[i] = 0.f;
   if (tid == 0) {
@@ -444,11 +450,9 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
             float swv[4]; // the node's face-node contributions (up to three faces meet at a node)
 #pragma unroll
             for (int n = 0; n < 4; ++n) {
-              swv[n] = 0.f;
-              uint32_t w = i + n < NP ? s_n2f[i + n] : 0xffffffffu;
-#pragma unroll
-              for (int j = 0; j < 3; ++j, w >>= 8)
-                if ((w & 0xffu) != 0xffu) swv[n] += s_x[(w & 0xffu) * T::RSX + ridx];
+              const uint32_t w = s_n2f[i + n < NP ? i + n : NP - 1];
+              const float *x = s_x + ridx;
+              swv[n] = x[(w & 0xffu) * T::RSX] + x[(w >> 8 & 0xffu) * T::RSX] + x[(w >> 16) * T::RSX];
             }
             const float4 lu4 = *reinterpret_cast<const float4 *>(s_lu + soff + i);
             const float4 lr4 = *reinterpret_cast<const float4 *>(s_lr + soff + i);
