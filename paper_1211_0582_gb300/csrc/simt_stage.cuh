@@ -219,8 +219,11 @@ __device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, 
       asm volatile("prefetch.global.L2 [%0];" ::"l"(u0 + c * KN + i));
       if (MODE != MODE_RHS && a.rk_a != 0.f) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.res + c * KN + k0 * NPP + i));
     }
-  // each field's value at the element's first node (see the volume term)
-  for (int i = tid; i < 6 * ne; i += NT) s_ref[i] = __ldcg(u0 + (i % 6) * KN + (i / 6) * NPP);
+  // each field's mean over the element's vertices (see the volume term)
+  for (int i = tid; i < 6 * ne; i += NT) {
+    const float *v = u0 + (i % 6) * KN + (i / 6) * NPP;
+    s_ref[i] = (0.25f * __ldcg(v) + 0.25f * __ldcg(v + N)) + (0.25f * __ldcg(v + NFP - 1) + 0.25f * __ldcg(v + NP - 1));
+  }
   cp_async_wait();
   __syncthreads();
 
