@@ -25,11 +25,11 @@
 // latencies of the traces and of the update that the blocks of an SM do not
 // cover for each other; at N <= 3 those latencies. Measured (us per stage
 // before, with three derivatives per field and the operators read through L1,
-// and now): N=1 162,000 tets 48.8 -> 33.4; N=2 131,712 tets 119 -> 73; N=3
-// 131,712 tets 203 -> 146; N=4 82,944 tets 298 -> 204; N=5 82,944 tets 479 ->
-// 394; N=6 24,576 tets 292 -> 227; N=7 24,576 tets 522 -> 422; N=8 24,576 tets
-// 859 -> 684; N=9 10,368 tets 668 -> 507; 162 tets at N=3 14.8 -> 6.6, 1,296
-// tets at N=5 21.1 -> 17.
+// and now): N=1 162,000 tets 48.8 -> 34.0; N=2 131,712 tets 119 -> 73; N=3
+// 131,712 tets 203 -> 145; N=4 82,944 tets 298 -> 206; N=5 82,944 tets 479 ->
+// 395; N=6 24,576 tets 292 -> 227; N=7 24,576 tets 522 -> 422; N=8 24,576 tets
+// 859 -> 685; N=9 10,368 tets 668 -> 507; 162 tets at N=3 14.8 -> 6.6, 1,296
+// tets at N=5 21.1 -> 14.4.
 #pragma once
 #include <atomic>
 #include <cmath>
@@ -219,11 +219,6 @@ __device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, 
       asm volatile("prefetch.global.L2 [%0];" ::"l"(u0 + c * KN + i));
       if (MODE != MODE_RHS && a.rk_a != 0.f) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.res + c * KN + k0 * NPP + i));
     }
-  // each field's mean over the element's vertices (see the volume term)
-  for (int i = tid; i < 6 * ne; i += NT) {
-    const float *v = u0 + (i % 6) * KN + (i / 6) * NPP;
-    s_ref[i] = (0.25f * __ldcg(v) + 0.25f * __ldcg(v + N)) + (0.25f * __ldcg(v + NFP - 1) + 0.25f * __ldcg(v + NP - 1));
-  }
   cp_async_wait();
   __syncthreads();
 
@@ -238,6 +233,23 @@ __device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, 
   for (int p = 0; p < 3 * RE; ++p)
 #pragma unroll
     for (int n = 0; n < 4 * CQ; ++n) acc[p][n] = make_float2(0.f, 0.f);
+
+  // Each field's mean over the element's vertices (see the volume term), or at
+  // N <= 3, where four scattered loads cost 2-3% of a stage, over its first
+  // four nodes. Taken after the first traces: by then the prefetched rows are
+  // in L2. With one chunk of face nodes the loads go ahead of the traces.
+  constexpr int RIT = (6 * Cfg::EB + NT - 1) / NT;
+  auto reference_nodes = [&](int i) {
+    const float *v = u0 + (i % 6) * KN + (i / 6) * NPP;
+    if constexpr (N <= 3) return load_field4(v);
+    else return make_float4(__ldcg(v), __ldcg(v + N), __ldcg(v + NFP - 1), __ldcg(v + NP - 1));
+  };
+  float4 rn[RIT];
+  if constexpr (FR >= D::NFF) {
+#pragma unroll
+    for (int t = 0; t < RIT; ++t)
+      if (tid + t * NT < 6 * ne) rn[t] = reference_nodes(tid + t * NT);
+  }
 
   // ---- flux gather and lifting, FR face nodes of every element at a time:
   // both traces from L2, the mirror state on walls; upwind flux with the
@@ -284,6 +296,15 @@ __device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, 
         d[2] = make_float2(fl[4], fl[5]);
       }
     }
+    if (r0 == 0) {
+#pragma unroll
+      for (int t = 0; t < RIT; ++t) {
+        const int i = tid + t * NT;
+        if (i >= 6 * ne) break;
+        if constexpr (FR < D::NFF) rn[t] = reference_nodes(i);
+        s_ref[i] = (0.25f * rn[t].x + 0.25f * rn[t].y) + (0.25f * rn[t].z + 0.25f * rn[t].w);
+      }
+    }
     cp_async_wait();
     __syncthreads();
     if (worker) simt_product<Cfg>(acc, xr, wr, fr);
@@ -291,11 +312,12 @@ __device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, 
 
   // ---- volume term, QC node quads at a time: the combinations of the curl
   // (d/dx_l = sum_d (dr_d/dx_l) d/dr_d) of every node and direction, then
-  // their derivatives. The fields enter as differences from their value at the
-  // element's first node: D annihilates constants, and without the constant
-  // part neither the rounded combinations nor the sums carry its rounding
-  // error (right-hand side at N=5 against 64 bits: 1.5e-6 with it, 9.5e-7
-  // without; 8.7e-7 with the combinations taken after the differentiation).
+  // their derivatives. The fields enter as differences from a mean of
+  // the element's: D annihilates constants, and without the constant part
+  // neither the rounded combinations nor the sums carry its rounding error
+  // (right-hand side at N=5 against 64 bits: 1.5e-6 with it, 9.5e-7 with
+  // differences from one node, 5.1e-7 now; 8.7e-7 with the combinations taken
+  // after the differentiation; N=3: 3.7e-7, 2.6e-7 now and 3.1e-7).
 #pragma unroll 1
   for (int q0 = 0; q0 < NQ; q0 += QC) {
     __syncthreads(); // the previous product has read X and the operator rows
