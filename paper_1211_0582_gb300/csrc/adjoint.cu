@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(AdjCfg<N>::NT2) k_adj_vol(AdjArgs a) {
     if (GRAD) {
       float qm[6], qp[6];
 #pragma unroll
-      for (int c = 0; c < 6; ++c) qm[c] = __ldg(a.u_s + c * KN + k * NPP + vm);
+      for (int c = 0; c < 6; ++c) qm[c] = a.u_s[c * KN + k * NPP + vm];
       if (wall) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(AdjCfg<N>::NT2) k_adj_vol(AdjArgs a) {
       } else {
         const int vn = s_nb[cny * NFP + m];
 #pragma unroll
-        for (int c = 0; c < 6; ++c) qp[c] = __ldg(a.u_s + c * KN + k2 * NPP + vn);
+        for (int c = 0; c < 6; ++c) qp[c] = a.u_s[c * KN + k2 * NPP + vn];
       }
       contrib = fnode.gradient(qm, qp, Z2, Y2, zs, ys, a.alpha, r2.y, r2.z);
     }

@@ -364,9 +364,9 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
         for (int c = 0; c < 6; ++c) g2[c] = wall ? 0.f : a.g[(c * a.K + k2) * NFF + fm2];
         if (grad) {
 #pragma unroll
-          for (int c = 0; c < 6; ++c) qm[c] = __ldg(a.u_s + c * KN + k * NPP + vm);
+          for (int c = 0; c < 6; ++c) qm[c] = a.u_s[c * KN + k * NPP + vm];
 #pragma unroll
-          for (int c = 0; c < 6; ++c) qp[c] = wall ? 0.f : __ldg(a.u_s + c * KN + k2 * NPP + vn);
+          for (int c = 0; c < 6; ++c) qp[c] = wall ? 0.f : a.u_s[c * KN + k2 * NPP + vn];
         }
         if (wall) {
 #pragma unroll

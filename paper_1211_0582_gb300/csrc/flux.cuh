@@ -18,7 +18,13 @@ struct Dims {
   static constexpr int NFF = 4 * NFP;                        // face nodes per element
 };
 
+// Loads of four floats: of data that no kernel of a launch chain writes
+// (operators), through the non-coherent path; of fields, plain. A stage is
+// resident while the stage before it still writes its fields (programmatic
+// dependent launch): ld.global.nc is not specified for such memory, a plain load
+// after griddepcontrol.wait is, and L1 holds its lines alike.
 __device__ __forceinline__ float4 ldg4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 
 // Flux difference n.(F - F*) at one face node, times Fscale (Section 5,
 // Fig. flux-code a, with jumps dq = q+ - q- and impedance weights for

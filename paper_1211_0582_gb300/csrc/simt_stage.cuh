@@ -104,14 +104,15 @@ struct SimtCfg {
 };
 
 // Field loads. Tile rows come from L2 past L1 (used once or twice); the face
-// nodes' scattered reads hit the same lines again and go through L1. A
-// persistent multi-stage launch (COHERENT) reads everything from L2: other
-// blocks wrote the data in an earlier stage.
+// nodes' scattered reads hit the same lines again and go through L1, as plain
+// loads (the previous stage writes these rows while this one is resident: see
+// ld4). A persistent multi-stage launch (COHERENT) reads everything from L2:
+// other blocks wrote the data in an earlier stage.
 __device__ __forceinline__ float4 load_field4(const float *p) { return __ldcg(reinterpret_cast<const float4 *>(p)); }
 template <bool COHERENT>
 __device__ __forceinline__ float load_trace(const float *p) {
   if constexpr (COHERENT) return __ldcg(p);
-  else return __ldg(p);
+  else return *p;
 }
 
 // The node tables of a block (once per launch; the first tile's barrier orders them).

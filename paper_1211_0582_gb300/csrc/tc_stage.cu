@@ -466,7 +466,7 @@ __global__ void __launch_bounds__(ENS ? 512 : TC<N>::THREADS, ENS ? 1 : TC<N>::B
                 } else {
                   const float *up = a.u + int64_t(cn.x) * NPP + node;
 #pragma unroll
-                  for (int c = 0; c < 6; ++c) qp[s][h][c] = ENS ? __ldcg(up + c * KN) : __ldg(up + c * KN);
+                  for (int c = 0; c < 6; ++c) qp[s][h][c] = ENS ? __ldcg(up + c * KN) : up[c * KN];
                 }
               }
             }
@@ -1223,7 +1223,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                   } else {
                     const float *up = a.u + int64_t(cn.x) * NPP + node;
 #pragma unroll
-                    for (int c = 0; c < 6; ++c) qp[ss][h][c] = __ldg(up + c * KN);
+                    for (int c = 0; c < 6; ++c) qp[ss][h][c] = up[c * KN];
                   }
                 }
               }

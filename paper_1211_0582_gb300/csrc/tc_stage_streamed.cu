@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(kThreadsS, 1)
       const int k = kq1 + 16 * s;
       v[s] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (cr1 >= 0 && k < NPP && e1 < ne) {
-        v[s] = ldg4(a.u + f1 * KN + (k0 + e1) * NPP + k);
+        v[s] = ld4(a.u + f1 * KN + (k0 + e1) * NPP + k);
         if (k + 3 >= NP) {
           if (k + 0 >= NP) v[s].x = 0.f;
           if (k + 1 >= NP) v[s].y = 0.f;
@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(kThreadsS, 1)
                 } else {
                   const float *up = a.u + int64_t(k2) * NPP + node;
 #pragma unroll
-                  for (int c = 0; c < 6; ++c) qp[b][h][c] = __ldg(up + c * KN);
+                  for (int c = 0; c < 6; ++c) qp[b][h][c] = up[c * KN];
                 }
               }
             }
@@ -562,8 +562,8 @@ __global__ void __launch_bounds__(kThreadsS, 1)
       // (the first LSERK4 stage has a = 0: the residual it overwrites is not read)
       if (MODE != MODE_LSERK || a.rk_a == 0.f || !live || ch >= ch1) return;
       const float *rp = a.res + fld * KN + k * NPP + ch * 8;
-      r0 = ldg4(rp);
-      if (ch * 8 + 4 < NPP) r1 = ldg4(rp + 4);
+      r0 = ld4(rp);
+      if (ch * 8 + 4 < NPP) r1 = ld4(rp + 4);
     };
     float4 rn0, rn1;
     load_res(ch0, rn0, rn1);
