@@ -648,7 +648,10 @@ cudaError_t launch_adj_tc_order(const AdjArgs &a, const AdjTcState &st, long lon
   const int tmem_fit = 512 / T::TCOLS;
   if (per_sm > tmem_fit) per_sm = tmem_fit;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const int cap = small_mesh_blocks<T::TE>(a.K, per_sm * st.sms);
+  // (half of the blocks on small meshes; at N = 5, one block per SM, up to 10
+  // elements per tile: a gradient's stage, us, all blocks and half: FP16x3 400 tets
+  // 31.1 -> 28.9, 1,300 tets 36.4 -> 38.0)
+  const int cap = small_mesh_blocks<T::TE>(a.K, per_sm * st.sms, N == 5 ? 10 : T::TE);
   const TileMap<T::TE> tm = make_tiles<T::TE>(a.K, cap);
   const int grid = tm.ntiles < cap ? tm.ntiles : cap;
   return launch_pdl(kern, dim3(unsigned(grid)), dim3(T::NT), size_t(T::SMEM), s, a,

@@ -425,6 +425,22 @@ __global__ void __launch_bounds__(SimtCfg<N, SMALL>::NT, SimtCfg<N, SMALL>::MINB
   }
 }
 
+// Blocks of a launch with room for `cap`: half of them on small meshes
+// (small_mesh_blocks), as far as that gains. It stops gaining at 20 elements per
+// tile at N = 1 (us per stage, all blocks and half: 6,080 tets 5.15 -> 4.74, 8,360
+// tets 5.33 -> 5.81), and where the larger tile's products take twice the warps: at
+// N = 3 beyond 6 elements (1,368 tets 7.40 -> 7.14, 1,482 tets 7.45 -> 8.17), at
+// N = 4 where the tiles of all blocks have 2, 6 or 8 elements (798 tets 9.33 ->
+// 10.05, 2,622 tets 12.1 -> 13.0; but 1,026 tets 11.4 -> 10.2, 2,964 tets 14.8 ->
+// 13.6). At the other orders it gains as far as half of the blocks hold the mesh
+// in full tiles (N=2 3,040 tets 7.12 -> 5.88, 7,296 tets 8.76 -> 8.22, though 3,344
+// tets 6.62 -> 6.96; N=5 2,432 tets 18.5 -> 15.7; N=8 912 tets 53.7 -> 35.1).
+template <int N, class Cfg>
+int simt_blocks(int64_t K, int cap) {
+  if (N == 4 && (K + cap - 1) / cap % 4 == 2) return cap;
+  return small_mesh_blocks<Cfg::EB>(K, cap, N == 1 ? 20 : N == 3 ? 6 : N == 4 ? 14 : Cfg::EB);
+}
+
 template <int N, int MODE, bool SMALL>
 cudaError_t launch_simt_mode(const StageArgs &a, int dev, int sms, cudaStream_t s) {
   using Cfg = SimtCfg<N, SMALL>;
@@ -443,7 +459,7 @@ cudaError_t launch_simt_mode(const StageArgs &a, int dev, int sms, cudaStream_t 
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     if (dev < kDevCache) per_sm_cache[dev].store(per_sm, std::memory_order_relaxed);
   }
-  const int cap = small_mesh_blocks<Cfg::EB>(a.K, per_sm * sms);
+  const int cap = simt_blocks<N, Cfg>(a.K, per_sm * sms);
   const TileMap<Cfg::EB> tm = make_tiles<Cfg::EB>(a.K, cap);
   const unsigned blocks = unsigned(tm.ntiles < cap ? tm.ntiles : cap);
   return launch_pdl(kern, dim3(blocks), dim3(Cfg::NT), Cfg::SMEM, s, a, tm);

@@ -1493,7 +1493,7 @@ cudaError_t launch_tc_kernel(const StageArgs &a, const TcState &st, int *flag, c
   if (e != cudaSuccess) return e;
   // with several blocks per SM, a mesh of at most one tile per SM is spread over
   // the SMs, not over their blocks
-  const int blocks = T::BLOCKS == 1 ? small_mesh_blocks<kTileElems>(a.K, st.sms)
+  const int blocks = T::BLOCKS == 1 ? small_mesh_blocks<kTileElems>(a.K, st.sms, MODE == MODE_RHS ? 12 : kTileElems)
                      : a.K <= int64_t(kTileElems) * st.sms ? st.sms : T::BLOCKS * st.sms;
   const TileMap<kTileElems> tm = make_tiles<kTileElems>(a.K, blocks);
   const int grid = tm.ntiles < blocks ? tm.ntiles : blocks;

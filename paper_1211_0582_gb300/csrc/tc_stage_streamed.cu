@@ -721,7 +721,7 @@ cudaError_t launch_streamed_kernel(const StageArgs &a, const TcState &st, int *f
   auto kern = k_stage_tc_streamed<N, MODE, BF16>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM);
   if (e != cudaSuccess) return e;
-  const int blocks = small_mesh_blocks<kTileS>(a.K, st.sms);
+  const int blocks = small_mesh_blocks<kTileS>(a.K, st.sms, 12);
   const TileMap<kTileS> tm = make_tiles<kTileS>(a.K, blocks);
   const int grid = tm.ntiles < blocks ? tm.ntiles : blocks;
   return launch_pdl(kern, dim3(unsigned(grid)), dim3(kThreadsS), size_t(T::SMEM), s, a,

@@ -35,16 +35,20 @@ TileMap<FULL> make_tiles(int64_t K, int grid) {
   return TileMap<FULL>{int(nfull), int(small), int(nfull + nsmall)};
 }
 
-// Blocks of a launch that may have `cap` resident at once: half of them where the
-// mesh fits half of them in full tiles. The other half of the SMs' room then
+// Blocks of a launch that may have `cap` resident at once: half of them where
+// their tiles then have at most `most` elements. The other half of the SMs' room
 // takes the next stage's blocks, whose setup (operators, tables, tensor memory)
-// overlaps this stage (programmatic dependent launch) instead of following it.
-// (us per stage, all blocks and half: FP16x3 N=4 1,296 tets 7.13 -> 6.72, N=5 750
-// tets 8.86 -> 7.11, N=7 162 tets 13.6 -> 12.9; FP32 N=3 1,296 tets 8.4 -> 7.4,
-// N=8 750 tets 54.6 -> 34.9; a few sizes at N <= 4 lose up to 9%.)
+// overlaps this stage (programmatic dependent launch) instead of following it;
+// in the FP32 stage a block that has its SM to itself is also through its tile
+// sooner. `most` is where each launch stops gaining, from sweeps over every tile
+// size (us per stage, all blocks and half): FP16x3 N=4 1,520 tets 7.37 -> 6.79,
+// N=5 1,520 tets 9.73 -> 8.01; N=7 912 tets 15.3 -> 15.1, but 1,520 tets 16.3 ->
+// 17.3: 12 elements at N = 6, 7. A right-hand side has no stage after it: on its
+// own it takes the same time either way up to 12 elements and longer from there
+// (FP16x3 N=4 760 tets 11.0 and 11.1, 1,216 tets 11.1 -> 12.6).
 template <int FULL>
-int small_mesh_blocks(int64_t K, int cap) {
-  return cap >= 2 && K <= int64_t(FULL) * (cap / 2) ? cap / 2 : cap;
+int small_mesh_blocks(int64_t K, int cap, int most = FULL) {
+  return cap >= 2 && K <= int64_t(most) * (cap / 2) ? cap / 2 : cap;
 }
 
 } // namespace dgmx
