@@ -45,19 +45,19 @@ __global__ void __launch_bounds__(Cfg::NT, Cfg::MINB)
 
 namespace dgmx {
 
-// Tile candidates of the autotuner for order N, in elements: where the small
-// shape serves alone its tile and three, two and one quarter of it; elsewhere
-// the two-element shape's tile and half of it, and the small shape's.
+// Tile candidates of the autotuner for order N, in elements: where the
+// one-element shape serves alone its tile and three, two and one quarter of it;
+// elsewhere the two-element shape's tile and half of it, and the one-element shape's.
 template <int N>
 struct EnsembleCandidates {
-  static constexpr bool small(int i) { return simt_small_only<N>() || i >= 2; }
+  static constexpr int shape(int i) { return simt_one_only<N>() || i >= 2 ? SHAPE_ONE : SHAPE_TWO; }
   static constexpr int c(int i) {
-    if (simt_small_only<N>()) return SimtShape<N, true>::EB * (4 - i) / 8 * 2;
-    const int step = i < 2 ? 4 : 2, eb = i < 2 ? SimtShape<N, false>::EB : SimtShape<N, true>::EB;
+    if (simt_one_only<N>()) return SimtShape<N, SHAPE_ONE>::EB * (4 - i) / 8 * 2;
+    const int step = i < 2 ? 4 : 2, eb = i < 2 ? SimtShape<N, SHAPE_TWO>::EB : SimtShape<N, SHAPE_ONE>::EB;
     return i % 2 ? eb / (2 * step) * step : eb;
   }
   template <int I>
-  using Cfg = SimtCfg<N, small(I), c(I)>;
+  using Cfg = SimtCfg<N, shape(I), c(I)>;
 };
 
 // occ = 0: as many blocks per SM as fit; occ = 1: half as many (rounded up),

@@ -42,40 +42,49 @@ namespace dgmx {
 
 // Shape of a launch: elements per tile and products per thread, RE elements x
 // CQ node quads (6 RE x 4 CQ accumulators).
-//   SMALL: one element x one quad and few, long chunks. A thread's chain of
+//   ONE: one element x one quad and few, long chunks. A thread's chain of
 //     products and a tile's chain of barriers are short, which is what counts
 //     while a launch has only a few tiles per SM; at N <= 3 and N = 6 it is
 //     the faster one at every size.
-//   otherwise two elements x two quads: half the shared-memory reads per
-//     product, but a tile takes as long with one element as with all of them.
-template <int N, bool SMALL>
+//   ONE_WIDE: the same with two or more times the elements per block (the rule is
+//     at simt_shape): more elements per SM in one round (N = 5: 36 instead of
+//     32), one copy of the operators for all of them.
+//   TWO: two elements x two quads: half the shared-memory reads per product, but
+//     a tile takes as long with one element as with all of them.
+enum SimtShapeKind { SHAPE_TWO = 0, SHAPE_ONE = 1, SHAPE_ONE_WIDE = 2 };
+template <int N, int SHAPE>
 struct SimtShape {
   using D = Dims<N>;
-  static constexpr int RE = SMALL ? 1 : 2, CQ = SMALL ? 1 : 2;
+  static constexpr bool ONE = SHAPE != SHAPE_TWO;
+  static constexpr int RE = ONE ? 1 : 2, CQ = ONE ? 1 : 2;
   static constexpr int CG = (D::NQ + CQ - 1) / CQ; // column groups: node quads cg and (CQ = 2) cg + CG
   // element groups of a block (even: neighbouring lanes hold two of them)
-  static constexpr int GROUPS = SMALL ? (N == 1 ? 64 : N <= 3 ? 32 : N == 4 ? 16 : N == 5 || N == 7 ? 8 : N == 6 ? 12
-                                         : N == 8 ? 6 : 4)
-                                      : 128 / CG / 2 * 2;
+  static constexpr int GROUPS = SHAPE == SHAPE_TWO        ? 128 / CG / 2 * 2
+                                : SHAPE == SHAPE_ONE_WIDE ? (N == 5 ? 18 : N == 7 ? 16 : N == 8 ? 12 : 8)
+                                : N == 1 ? 64 : N <= 3 ? 32 : N == 4 ? 16 : N == 6 ? 12 : N == 8 ? 6 : N == 9 ? 4 : 8;
   static constexpr int EB = RE * GROUPS;
   // Rows of X per chunk: FR face nodes (even, as 4 Nfp is) or QC node quads
   // (12 rows each).
-  static constexpr int FR = SMALL ? (N == 9 ? 44 : N == 8 ? 60 : N == 7 ? 72 : D::NFF)
+  static constexpr int FR = ONE ? (N == 9 ? 44 : N == 8 ? 60 : N == 7 ? 72 : D::NFF)
                                   : N == 9 ? 44 : N == 8 ? 60 : N == 7 ? 72 : N == 5 ? 42 : 30;
-  static constexpr int QC = SMALL ? (N == 9 ? 5 : N == 8 ? 7 : N == 7 ? 6 : N == 6 || N == 5 ? 7 : D::NQ)
+  static constexpr int QC = ONE ? (N == 9 ? 5 : N == 8 ? 7 : N == 7 ? 6 : N == 6 || N == 5 ? 7 : D::NQ)
                                   : N == 9 ? 4 : N == 8 ? 5 : N == 7 ? 6 : N == 5 ? 4 : 2;
 };
 
-// Orders that only the small shape serves.
+// Orders that only the first shape serves, and those with the wide one.
 template <int N>
-constexpr bool simt_small_only() {
+constexpr bool simt_one_only() {
   return N <= 3 || N == 6;
 }
+template <int N>
+constexpr bool simt_has_wide() {
+  return N == 5 || N >= 7;
+}
 
-template <int N, bool SMALL, int EB_ = SimtShape<N, SMALL>::EB>
+template <int N, int SHAPE, int EB_ = SimtShape<N, SHAPE>::EB>
 struct SimtCfg {
   using D = Dims<N>;
-  using S = SimtShape<N, SMALL>;
+  using S = SimtShape<N, SHAPE>;
   static constexpr int EB = EB_;
   static_assert(EB % (2 * S::RE) == 0 && EB <= S::EB, "whole pairs of element groups");
   static constexpr int QC = S::QC, FR = S::FR, CG = S::CG;
@@ -96,10 +105,10 @@ struct SimtCfg {
   static constexpr int OFF_REF = OFF_G + EB * GS * 4;  // float [EB][6]
   static constexpr int OFF_TAB = OFF_REF + EB * 24;
   static constexpr size_t SMEM = size_t(OFF_TAB + (100 * D::NFP + 15) / 16 * 16);
-  // blocks per SM asked for: three of 168 registers per thread, or (SMALL) as
-  // many of 128 as shared memory holds
+  // blocks per SM asked for: three of 168 registers per thread, or (one element per
+  // thread) as many of 128 as shared memory holds
   static constexpr int FIT = int(228 * 1024 / (SMEM + 1024)) < 512 / NT ? int(228 * 1024 / (SMEM + 1024)) : 512 / NT > 0 ? 512 / NT : 1;
-  static constexpr int MINB = SMALL ? FIT : 3;
+  static constexpr int MINB = S::ONE ? FIT : 3;
   static_assert(SMEM <= 228 * 1024 / MINB - 1024, "MINB blocks per SM");
 };
 
@@ -408,9 +417,9 @@ __device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, 
   }
 }
 
-template <int N, int MODE, bool SMALL>
-__global__ void __launch_bounds__(SimtCfg<N, SMALL>::NT, SimtCfg<N, SMALL>::MINB) k_stage_simt(StageArgs a, TileMap<SimtCfg<N, SMALL>::EB> tm) {
-  using Cfg = SimtCfg<N, SMALL>;
+template <int N, int MODE, int SHAPE>
+__global__ void __launch_bounds__(SimtCfg<N, SHAPE>::NT, SimtCfg<N, SHAPE>::MINB) k_stage_simt(StageArgs a, TileMap<SimtCfg<N, SHAPE>::EB> tm) {
+  using Cfg = SimtCfg<N, SHAPE>;
   extern __shared__ float4 smem4[];
   simt_setup<Cfg>(a, smem4);
   // (the operator is fixed: its first rows may arrive before the previous stage has ended)
@@ -441,10 +450,10 @@ int simt_blocks(int64_t K, int cap) {
   return small_mesh_blocks<Cfg::EB>(K, cap, N == 1 ? 20 : N == 3 ? 6 : N == 4 ? 14 : Cfg::EB);
 }
 
-template <int N, int MODE, bool SMALL>
+template <int N, int MODE, int SHAPE>
 cudaError_t launch_simt_mode(const StageArgs &a, int dev, int sms, cudaStream_t s) {
-  using Cfg = SimtCfg<N, SMALL>;
-  auto kern = k_stage_simt<N, MODE, SMALL>;
+  using Cfg = SimtCfg<N, SHAPE>;
+  auto kern = k_stage_simt<N, MODE, SHAPE>;
   // the shared-memory opt-in is a per-device function attribute: set it on every launch
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Cfg::SMEM));
   if (e != cudaSuccess) return e;
@@ -466,20 +475,43 @@ cudaError_t launch_simt_mode(const StageArgs &a, int dev, int sms, cudaStream_t 
 }
 
 // The two-element shape runs in rounds of one tile per block that take the same
-// time however many elements a tile has; the small shape's time grows with the
-// element count, by simt_round_ratio times a round's time per full round of
+// time however many elements a tile has; the one-element shape's time grows with
+// the element count, by simt_round_ratio times a round's time per full round of
 // elements (measured, us per round and us per full round's elements in the
-// small shape: N=4 50 / 61, N=5 63 / 85, N=7 103 / 128, N=8 134 / 181, N=9 168 /
-// 228). The first is taken where its rounds cost less.
+// one-element shape: N=4 50 / 61, N=5 63 / 85, N=7 103 / 128, N=8 134 / 181, N=9
+// 168 / 228). The first is taken where its rounds cost less.
+//
+// The wide one-element shape is taken where the narrow one's blocks no longer hold
+// the mesh in less than a round: beyond one block per SM at N >= 7, where a
+// second one on the SM takes turns with the first, and beyond half of the blocks at
+// N = 5, but not with six elements per narrow tile, which fill three warps (us per
+// stage, narrow and wide: N=5 2,700 tets 21.4 -> 16.6, 3,300 tets 21.7 -> 23.1, 5,300
+// tets 39.8 -> 26.7, 10,500 tets 66.1 -> 49.9; N=7 1,310 tets 39.7 -> 31.5; N=8 1,215
+// tets 54.8 -> 43.6, 2,535 tets 111 -> 88; N=9 670 tets 72.5 -> 56.5, 2,590 tets 189 ->
+// 170). At N >= 7 not where few elements are left after whole rounds: the narrow
+// blocks do those beside other blocks' full tiles (N=8 1,875 tets 69.5, wide 79.2;
+// 1,995 tets 92.1, wide 79.6).
 template <int N>
 constexpr double simt_round_ratio() {
   return N == 4 ? 1.22 : N == 7 ? 1.24 : 1.35;
 }
 template <int N>
-bool simt_small(int64_t K, int sms) {
-  if (simt_small_only<N>()) return true;
-  const double rounds = double(K) / (double(SimtCfg<N, false>::MINB) * sms * SimtShape<N, false>::EB);
-  return std::ceil(rounds) >= simt_round_ratio<N>() * rounds;
+int simt_shape(int64_t K, int sms) {
+  if constexpr (!simt_one_only<N>()) {
+    const double rounds = double(K) / (double(SimtCfg<N, SHAPE_TWO>::MINB) * sms * SimtShape<N, SHAPE_TWO>::EB);
+    if (std::ceil(rounds) < simt_round_ratio<N>() * rounds) return SHAPE_TWO;
+  }
+  if constexpr (simt_has_wide<N>()) {
+    using One = SimtCfg<N, SHAPE_ONE>;
+    const int64_t round = int64_t(One::EB) * (N == 5 ? One::MINB / 2 : 1) * sms;
+    const int64_t wide = int64_t(SimtShape<N, SHAPE_ONE_WIDE>::EB) * sms; // N >= 7: a round of the wide shape
+    if (K > round) {
+      if (N == 5) return (K - 1) / (int64_t(One::MINB) * sms) + 1 == 6 ? SHAPE_ONE : SHAPE_ONE_WIDE;
+      const int64_t left = K % wide;
+      if (left == 0 || 2 * left > sms) return SHAPE_ONE_WIDE;
+    }
+  }
+  return SHAPE_ONE;
 }
 
 template <int N, int MODE>
@@ -488,9 +520,12 @@ cudaError_t launch_simt_shape(const StageArgs &a, cudaStream_t s) {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  if constexpr (!simt_small_only<N>())
-    if (!simt_small<N>(a.K, sms)) return launch_simt_mode<N, MODE, false>(a, dev, sms, s);
-  return launch_simt_mode<N, MODE, true>(a, dev, sms, s);
+  const int shape = simt_shape<N>(a.K, sms);
+  if constexpr (!simt_one_only<N>())
+    if (shape == SHAPE_TWO) return launch_simt_mode<N, MODE, SHAPE_TWO>(a, dev, sms, s);
+  if constexpr (simt_has_wide<N>())
+    if (shape == SHAPE_ONE_WIDE) return launch_simt_mode<N, MODE, SHAPE_ONE_WIDE>(a, dev, sms, s);
+  return launch_simt_mode<N, MODE, SHAPE_ONE>(a, dev, sms, s);
 }
 
 template <int N>
