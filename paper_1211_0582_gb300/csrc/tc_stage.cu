@@ -245,8 +245,22 @@ __global__ void __launch_bounds__(ENS ? 512 : TC<N>::THREADS, ENS ? 1 : TC<N>::B
   // ---- one-time setup
   for (int i = tid; i < T::A2R / 16; i += NTH)
     reinterpret_cast<uint4 *>(smem + T::OFF_A2H)[i] = make_uint4(0u, 0u, 0u, 0u);
-  for (int i = tid; i < T::OPS_BYTES / 16; i += NTH)
-    reinterpret_cast<uint4 *>(smem + T::OFF_B1H)[i] = __ldg(ops + i);
+  // the operators; at N <= 3 all of a thread's loads are in flight together (one
+  // latency for 256 threads' loads; a lone right-hand side, us: FP16x3 N=3 3,000
+  // tets 12.0 -> 11.1, 9,000 tets 18.7 -> 17.2; BF16x3 N=3 100 tets 10.5 -> 9.8)
+  constexpr int OPL = T::OPS_BYTES / 16;
+  uint4 *s_ops = reinterpret_cast<uint4 *>(smem + T::OFF_B1H);
+  if constexpr (N <= 3) {
+    uint4 w[(OPL + NTH - 1) / NTH];
+#pragma unroll
+    for (int j = 0; j < (OPL + NTH - 1) / NTH; ++j)
+      if (tid + j * NTH < OPL) w[j] = __ldg(ops + tid + j * NTH);
+#pragma unroll
+    for (int j = 0; j < (OPL + NTH - 1) / NTH; ++j)
+      if (tid + j * NTH < OPL) s_ops[tid + j * NTH] = w[j];
+  } else {
+    for (int i = tid; i < OPL; i += NTH) s_ops[i] = __ldg(ops + i);
+  }
   for (int i = tid; i < NFF + kConnKinds * NFP; i += NTH)
     s_fm[i] = i < NFF ? a.fmask[i] : a.nbrtab[i - NFF];
   for (int i = tid; i < 256 + 2 * kTileElems; i += NTH) s_inv1[i] = i < 128 ? 1.f : 0.f;
@@ -434,6 +448,12 @@ __global__ void __launch_bounds__(ENS ? 512 : TC<N>::THREADS, ENS ? 1 : TC<N>::B
       TC_MARK(2);
 
       bool ok = true;
+      // does the warp's s-th flux block exist? At N <= 3, where a warp of 256
+      // threads has two, the second one is skipped where the tile does not reach
+      // it (its rows are not read): us per stage, FP16x3 N=2 300 tets 4.65 -> 4.50,
+      // N=3 162 tets 5.00 -> 4.91; testing the first one too costs full tiles 2%
+      const int nblk = (ne + 3) / 4 * KGF;
+      auto flux_block = [&](int s, int blk) { return blk < (N <= 3 && s > 0 ? nblk : NBLK); };
 
       // ---- 3. upwind flux, in registers: the neighbour traces
       // outside the tile are requested from L2 first (all of a lane's loads in
@@ -452,7 +472,7 @@ __global__ void __launch_bounds__(ENS ? 512 : TC<N>::THREADS, ENS ? 1 : TC<N>::B
 #pragma unroll
           for (int c = 0; c < 6; ++c) qp[s][h][c] = 0.f;
         }
-        if (blk < NBLK && f < 4 && e < ne) {
+        if (flux_block(s, blk) && f < 4 && e < ne) {
           const int2 cn = s_fconn[e * 4 + f];
           if (cn.y != kBoundaryConn) {
             const int el = cn.x - int(k0);
@@ -483,7 +503,7 @@ __global__ void __launch_bounds__(ENS ? 512 : TC<N>::THREADS, ENS ? 1 : TC<N>::B
         for (int h = 0; h < 2; ++h)
 #pragma unroll
           for (int c = 0; c < 6; ++c) fl[s][h][c] = 0.f;
-        if (blk < NBLK && f < 4 && e < ne) {
+        if (flux_block(s, blk) && f < 4 && e < ne) {
           const float4 g0 = s_fgeo[e * 4 + f], w1 = s_fmat[e * 4 + f];
           const bool wall = s_fconn[e * 4 + f].y == kBoundaryConn;
           {
@@ -518,7 +538,7 @@ __global__ void __launch_bounds__(ENS ? 512 : TC<N>::THREADS, ENS ? 1 : TC<N>::B
           // exponents of the lane's E and H fluxes packed into one word, the
           // bytewise maximum over the 8 lanes of the element, one
           // shared-memory maximum per element, type and block
-          if (blk < NBLK) { // warp-uniform
+          if (flux_block(s, blk)) { // warp-uniform
             uint32_t mE = 0u, mH = 0u;
 #pragma unroll
             for (int h = 0; h < 2; ++h)
@@ -587,7 +607,7 @@ __global__ void __launch_bounds__(ENS ? 512 : TC<N>::THREADS, ENS ? 1 : TC<N>::B
         for (int s = 0; s < R2; ++s) {
           const int blk = warp + NW * s;
           const int e = 4 * (blk / KGF) + eo, fm = 16 * (blk % KGF) + 2 * kp;
-          if (blk < NBLK) {
+          if (flux_block(s, blk)) {
             float sc2[6];
 #pragma unroll
             for (int c = 0; c < 6; ++c) sc2[c] = 1.f;
@@ -1491,10 +1511,13 @@ cudaError_t launch_tc_kernel(const StageArgs &a, const TcState &st, int *flag, c
   // the largest shared-memory carveout, so that the blocks of an SM fit side by side
   if (e == cudaSuccess && T::BLOCKS > 1) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   if (e != cudaSuccess) return e;
-  // with several blocks per SM, a mesh of at most one tile per SM is spread over
-  // the SMs, not over their blocks
+  // with several blocks per SM, as many of them as a round of full tiles needs: a
+  // mesh of at most one tile per SM is spread over the SMs, not over their blocks
+  // (us per stage, four blocks and now: FP16x3 N=1 3,600 tets 6.74 -> 4.57 with two,
+  // 9,000 tets 7.13 -> 6.17 with three)
+  const int64_t tiles_per_sm = (a.K + kTileElems * st.sms - 1) / (kTileElems * st.sms);
   const int blocks = T::BLOCKS == 1 ? small_mesh_blocks<kTileElems>(a.K, st.sms, MODE == MODE_RHS ? 12 : kTileElems)
-                     : a.K <= int64_t(kTileElems) * st.sms ? st.sms : T::BLOCKS * st.sms;
+                     : int(tiles_per_sm < T::BLOCKS ? tiles_per_sm : T::BLOCKS) * st.sms;
   const TileMap<kTileElems> tm = make_tiles<kTileElems>(a.K, blocks);
   const int grid = tm.ntiles < blocks ? tm.ntiles : blocks;
   return launch_pdl(kern, dim3(unsigned(grid)), dim3(T::THREADS), size_t(T::SMEM), s, a,
