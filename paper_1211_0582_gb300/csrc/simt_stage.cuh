@@ -63,8 +63,8 @@ struct SimtShape {
                                 : SHAPE == SHAPE_ONE_WIDE ? (N == 5 ? 18 : N == 7 ? 16 : N == 8 ? 12 : 8)
                                 : N == 1 ? 64 : N <= 3 ? 32 : N == 4 ? 16 : N == 6 ? 12 : N == 8 ? 6 : N == 9 ? 4 : 8;
   static constexpr int EB = RE * GROUPS;
-  // Rows of X per chunk: FR face nodes (even, as 4 Nfp is) or QC node quads
-  // (12 rows each).
+  // Rows of X per chunk: FR face nodes (even, a divisor of 4 Nfp) or QC node
+  // quads (12 rows each).
   static constexpr int FR = ONE ? (N == 9 ? 44 : N == 8 ? 60 : N == 7 ? 72 : D::NFF)
                                   : N == 9 ? 44 : N == 8 ? 60 : N == 7 ? 72 : N == 5 ? 42 : 30;
   static constexpr int QC = ONE ? (N == 9 ? 5 : N == 8 ? 7 : N == 7 ? 6 : N == 6 || N == 5 ? 7 : D::NQ)
@@ -88,6 +88,7 @@ struct SimtCfg {
   static constexpr int EB = EB_;
   static_assert(EB % (2 * S::RE) == 0 && EB <= S::EB, "whole pairs of element groups");
   static constexpr int QC = S::QC, FR = S::FR, CG = S::CG;
+  static_assert(D::NFF % FR == 0 && FR % 2 == 0, "whole chunks of face nodes, an even number of rows");
   static constexpr int NT = EB / S::RE * CG > 128 ? (EB / S::RE * CG + 31) / 32 * 32 : 128; // threads per block
   // Row stride of X: an odd multiple of 4 floats (16-byte loads along the rows
   // are aligned, the stores of neighbouring nodes fall into different banks)
@@ -213,7 +214,7 @@ __device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, 
   const int64_t KN = a.K * NPP;
   const float *u0 = a.u + k0 * NPP;
 
-  if (!staged) simt_stage_operator<Cfg>(s_w, a.LT, FR < D::NFF ? FR : D::NFF);
+  if (!staged) simt_stage_operator<Cfg>(s_w, a.LT, FR);
   for (int i = tid; i < ne * 4; i += NT) {
     cp_async<16>(s_fgeo + i, a.fgeo + k0 * 4 + i);
     cp_async<16>(s_fmat + i, a.fmat + k0 * 4 + i);
@@ -255,7 +256,7 @@ __device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, 
     else return make_float4(__ldcg(v), __ldcg(v + N), __ldcg(v + NFP - 1), __ldcg(v + NP - 1));
   };
   float4 rn[RIT];
-  if constexpr (FR >= D::NFF) {
+  if constexpr (FR == D::NFF) {
 #pragma unroll
     for (int t = 0; t < RIT; ++t)
       if (tid + t * NT < 6 * ne) rn[t] = reference_nodes(tid + t * NT);
@@ -267,8 +268,7 @@ __device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, 
 #pragma unroll 1
   for (int r0 = 0; r0 < D::NFF; r0 += FR) {
     if (r0) __syncthreads(); // the previous product has read X and the operator rows
-    const int fr = D::NFF % FR == 0 || D::NFF - r0 >= FR ? FR : D::NFF - r0;
-    if (r0) simt_stage_operator<Cfg>(s_w, a.LT + r0 * NPP, fr);
+    if (r0) simt_stage_operator<Cfg>(s_w, a.LT + r0 * NPP, FR);
     const int items = ne * FR;
     constexpr int B = 2;
 #pragma unroll 1
@@ -279,7 +279,7 @@ __device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, 
       for (int i = 0; i < B; ++i) {
         const int it = it0 + i * NT, e = it / FR, r = it - e * FR, fm = r0 + r, f = fm / NFP;
         wall[i] = false;
-        if (it < items && (D::NFF % FR == 0 || r < fr)) {
+        if (it < items) {
           const int2 cn = s_fconn[e * 4 + f];
           const float *um = u0 + e * NPP + s_fm[fm], *up = um;
           wall[i] = cn.y == kBoundaryConn;
@@ -293,7 +293,7 @@ __device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, 
 #pragma unroll
       for (int i = 0; i < B; ++i) {
         const int it = it0 + i * NT, e = it / FR, r = it - e * FR, fm = r0 + r, f = fm / NFP;
-        if (it >= items || (D::NFF % FR != 0 && r >= fr)) break;
+        if (it >= items) break;
         if (wall[i]) {
 #pragma unroll
           for (int c = 0; c < 3; ++c) qp[i][c] = -qm[i][c];
@@ -317,7 +317,7 @@ __device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, 
     }
     cp_async_wait();
     __syncthreads();
-    if (worker) simt_product<Cfg>(acc, xr, wr, fr);
+    if (worker) simt_product<Cfg>(acc, xr, wr, FR);
   }
 
   // ---- volume term, QC node quads at a time: the combinations of the curl
@@ -423,8 +423,7 @@ __global__ void __launch_bounds__(SimtCfg<N, SHAPE>::NT, SimtCfg<N, SHAPE>::MINB
   extern __shared__ float4 smem4[];
   simt_setup<Cfg>(a, smem4);
   // (the operator is fixed: its first rows may arrive before the previous stage has ended)
-  simt_stage_operator<Cfg>(reinterpret_cast<float *>(reinterpret_cast<uint8_t *>(smem4) + Cfg::OFF_W), a.LT,
-                           Cfg::FR < Cfg::D::NFF ? Cfg::FR : Cfg::D::NFF);
+  simt_stage_operator<Cfg>(reinterpret_cast<float *>(reinterpret_cast<uint8_t *>(smem4) + Cfg::OFF_W), a.LT, Cfg::FR);
   pdl_wait(); // stage after stage: fields of the previous stage from here on
   for (int t = blockIdx.x; t < tm.ntiles; t += gridDim.x) {
     if (t + int(gridDim.x) >= tm.ntiles) pdl_launch_next(); // this block's last tile
