@@ -204,8 +204,8 @@ int dg_mesh_upload(dg_ctx *ctx, int64_t Nv, const double *VX, const double *VY, 
   cudaStream_t s = ctx->stream;
 
   // host-side operator layouts for the CUDA-core kernels
-  // (rows read ahead of their use and past a row's end: three rows of padding)
-  std::vector<float> DT(size_t(3) * (Npad + 1) * Npad, 0.f), LT(size_t(4 * Nfp + 3) * Npad, 0.f);
+  // (whole node quads of D^T are staged: the rows of nodes Np to Npad - 1 are zeros)
+  std::vector<float> DT(size_t(3) * Npad * Npad, 0.f), LT(size_t(4) * Nfp * Npad, 0.f);
   const std::vector<double> *Ds[3] = {&o.Dr, &o.Ds, &o.Dt};
   for (int d = 0; d < 3; ++d)
     for (int j = 0; j < Np; ++j)

@@ -34,8 +34,8 @@ struct StageArgs {
   const int2 *fconn;   // [K][4] {neighbour element, connection kind}
   const float4 *fmat;  // [K][4] {Fscale/(Z-+Z+), -Fscale/(Y-+Y+), Z+, Y+} flux weights per face
   long long wait_limit; // device waits give up after this many SM cycles (0 = default, ~1 s)
-  const float *DT;     // [Npad + 1][3][Npad] transposed Dr, Ds, Dt per node (zero rows from node Np on)
-  const float *LT;     // [4Nfp + 3][Npad] transposed LIFT (three zero rows at the end)
+  const float *DT;     // [Npad][3][Npad] transposed Dr, Ds, Dt per node (zero rows from node Np on)
+  const float *LT;     // [4Nfp][Npad] transposed LIFT
   const uint8_t *fmask;  // [4Nfp]  volume node of each face node
   const uint8_t *nbrtab; // [96][Nfp] neighbour volume node per connection kind
   int64_t K;
