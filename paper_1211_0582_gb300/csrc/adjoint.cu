@@ -42,7 +42,7 @@ struct AdjCfg {
   static constexpr int EB2 = 80 / D::NQ > 0 ? 80 / D::NQ : 1; // elements per volume block (measured best)
   static constexpr int NT2 = (EB2 * D::NQ + 31) / 32 * 32;
   static constexpr size_t SMEM1 = size_t(6) * EB1 * D::NPP * 4;
-  static constexpr size_t SMEM2 = size_t(EB2) * 4 * 64 + (size_t(6) * EB2 * D::NPP * 2 + EB2) * 4 +
+  static constexpr size_t SMEM2 = size_t(EB2) * 4 * 48 + (size_t(6) * EB2 * D::NPP * 2 + EB2) * 4 +
                                   ((200 * D::NFP + 15) / 16) * 16;
 };
 
@@ -127,10 +127,10 @@ __global__ void __launch_bounds__(AdjCfg<N>::NT2) k_adj_vol(AdjArgs a) {
   constexpr int NP = D::NP, NPP = D::NPP, NQ = D::NQ, NFF = D::NFF, NFP = D::NFP, EB = C::EB2, NT = C::NT2;
   constexpr int MQ = C::MQ;
   extern __shared__ float4 smem4[];
-  // per face of the block's elements: {n, 1/(Z-+Z+)}, {Z-, Z+, Y-, Y+},
-  // {1/(Y-+Y+), dZ-/deps, dY-/deps, connection kind}, {neighbour element, wall}
-  float4 *s_face = smem4;                                 // [EB * 4][4]
-  float *s_v = reinterpret_cast<float *>(smem4 + EB * 16); // W lr   [6][EB][NPP]
+  // per face of the block's elements: {n, 1/(Z-+Z+)}, {Z+, Y+, 1/(Y-+Y+),
+  // connection kind}, {dZ-/deps, dY-/deps, neighbour element, 0}
+  float4 *s_face = smem4;                                 // [EB * 4][3]
+  float *s_v = reinterpret_cast<float *>(smem4 + EB * 12); // W lr   [6][EB][NPP]
   float *s_w = s_v + 6 * EB * NPP;               // surface contributions [6][EB][NPP]
   float *s_gr = s_w + 6 * EB * NPP;              // gradient partial per element [EB]
   uint8_t *s_fm = reinterpret_cast<uint8_t *>(s_gr + EB);
@@ -153,10 +153,9 @@ __global__ void __launch_bounds__(AdjCfg<N>::NT2) k_adj_vol(AdjArgs a) {
     const int64_t k2 = wall ? k : cn.x;
     const float Z2 = wall ? Zk : __ldg(a.geo + k2 * G_STRIDE + G_Z), Y2 = wall ? Yk : __ldg(a.geo + k2 * G_STRIDE + G_Y);
     const float ek = 1.f / __ldg(a.geo + k * G_STRIDE + G_IEPS);
-    s_face[t * 4 + 0] = make_float4(nf.x, nf.y, nf.z, 1.f / (Zk + Z2));
-    s_face[t * 4 + 1] = make_float4(Zk, Z2, Yk, Y2);
-    s_face[t * 4 + 2] = make_float4(1.f / (Yk + Y2), -Zk / (2.f * ek), Yk / (2.f * ek), __int_as_float(cn.y));
-    s_face[t * 4 + 3] = make_float4(__int_as_float(int(k2)), __int_as_float(wall ? 1 : 0), 0.f, 0.f);
+    s_face[t * 3 + 0] = make_float4(nf.x, nf.y, nf.z, 1.f / (Zk + Z2));
+    s_face[t * 3 + 1] = make_float4(Z2, Y2, 1.f / (Yk + Y2), __int_as_float(cn.y));
+    s_face[t * 3 + 2] = make_float4(-Zk / (2.f * ek), Yk / (2.f * ek), __int_as_float(int(k2)), 0.f);
   }
   // the tables and face constants above are static: the previous kernel's
   // results (lambda, face data, gradient) are read from here on
@@ -208,13 +207,13 @@ __global__ void __launch_bounds__(AdjCfg<N>::NT2) k_adj_vol(AdjArgs a) {
     const int64_t k = k0 + e;
     float contrib = 0.f;
     if (it < EB * NFF && k < a.K) {
-    const float4 *fr = s_face + (e * 4 + f) * 4;
-    const float4 r0 = fr[0], r1 = fr[1], r2 = fr[2], r3 = fr[3];
+    const float4 *fr = s_face + (e * 4 + f) * 3;
+    const float4 r0 = fr[0], r1 = fr[1], r2 = fr[2];
     const float n[3] = {r0.x, r0.y, r0.z};
-    const float zs = r0.w, Z2 = r1.y, Y2 = r1.w, ys = r2.x;
-    const int cny = __float_as_int(r2.w);
-    const int64_t k2 = __float_as_int(r3.x);
-    const bool wall = __float_as_int(r3.y) != 0;
+    const float zs = r0.w, Z2 = r1.x, Y2 = r1.y, ys = r1.z;
+    const int cny = __float_as_int(r1.w);
+    const int64_t k2 = __float_as_int(r2.z);
+    const bool wall = cny == kBoundaryConn;
     float gk[6];
 #pragma unroll
     for (int c = 0; c < 6; ++c) gk[c] = a.g[(c * a.K + k) * NFF + fm];
@@ -246,7 +245,7 @@ __global__ void __launch_bounds__(AdjCfg<N>::NT2) k_adj_vol(AdjArgs a) {
 #pragma unroll
         for (int c = 0; c < 6; ++c) qp[c] = a.u_s[c * KN + k2 * NPP + vn];
       }
-      contrib = fnode.gradient(qm, qp, Z2, Y2, zs, ys, a.alpha, r2.y, r2.z);
+      contrib = fnode.gradient(qm, qp, Z2, Y2, zs, ys, a.alpha, r2.x, r2.y);
     }
     }
     if (GRAD) add_by_element(s_gr, e, contrib);
@@ -738,7 +737,7 @@ int dg_adjoint_step(dg_ctx *ctx, const float *u0, const float *eps, double dt, i
   // where supported unless the CUDA-core form was asked for; that form reads
   // per-face constants computed once per call
   const bool tc_reverse = ctx->adj_form != 0 && adj_tc_supported(ctx);
-  float4 *fcon = tc_reverse ? ws.get<float4>(17, size_t(16) * ctx->K) : nullptr;
+  float4 *fcon = tc_reverse ? ws.get<float4>(17, size_t(12) * ctx->K) : nullptr;
   if (tc_reverse && !fcon) return fail(ctx, DG_ERR_OOM, "dg_adjoint_step: device allocation failed (face constants)");
   // stage states u_s and the E components of the stage right-hand sides A u_s of one segment
   float *US = ws.get<float>(10, fl * 5 * C), *RS = ws.get<float>(11, hfl * 5 * C);

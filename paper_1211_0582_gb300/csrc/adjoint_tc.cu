@@ -28,8 +28,10 @@
 // lambda_u, the E rows of the stage's right-hand side, its face data and
 // per-face constants arrive by bulk copies (requested during the previous
 // tile); W lr is split into the A operand of GEMM-D in tensor memory; while
-// GEMM-D runs, the face loop scatters the transposed flux into a shared-memory
-// buffer; the epilogue forms lambda_u + dt (curl^T + flux^T), the next stage's
+// GEMM-D runs, the face loop stores what each face node contributes to its volume
+// node, per face node, over the E rows of the right-hand side, which have been
+// read by then; the epilogue gathers a node's up to three contributions, forms
+// lambda_u + dt (curl^T + flux^T), the next stage's
 // lambda_r = a lambda_r + b_next lambda_u and its split W lr' (over the
 // columns of T, which have been read); GEMM-L lifts it, and the face data
 // g_next = Fscale G go to global memory. Two blocks per SM at N <= 4 overlap
@@ -107,9 +109,9 @@ struct AT {
   static_assert(NFF < 255, "face nodes are bytes");
   static constexpr int OFF_X = OFF_LU + TB, OFF_RS = OFF_X;
   static constexpr int ZROW = rup(XB, 4 * RSX) / (4 * RSX); // a row of zeros past the buffer
-  static constexpr int OFF_FACE = OFF_X + rup((ZROW + 1) * RSX * 4, 128); // float4 [80][4] per-face constants
+  static constexpr int OFF_FACE = OFF_X + rup((ZROW + 1) * RSX * 4, 128); // float4 [80][3] per-face constants
   static_assert(ZROW < 255, "row numbers are bytes");
-  static constexpr int OFF_FG = OFF_FACE + kAdjTile * 4 * 64; // float4 [80] {n, Fscale}
+  static constexpr int OFF_FG = OFF_FACE + kAdjTile * 4 * 48; // float4 [80] {n, Fscale}
   static constexpr int OFF_GEO = OFF_FG + kAdjTile * 4 * 16;  // float [20][G_STRIDE]
   static constexpr int OFF_TAB = OFF_GEO + kAdjTile * G_STRIDE * 4;
   // u32 [128] row maxima, float [128] inverse row scales, float [20] gradient partials
@@ -240,10 +242,10 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
   auto stage_faces = [&](int t) {
     const int64_t kb = tm.start(t);
     const uint32_t nb = uint32_t(tm.size(t, a.K));
-    umma::mbar_arrive_expect_tx(barF, nb * (64u + G_STRIDE * 4u + 256u));
+    umma::mbar_arrive_expect_tx(barF, nb * (64u + G_STRIDE * 4u + 192u));
     umma::bulk_g2s(smem + T::OFF_FG, a.fgeo + kb * 4, nb * 64u, barF);
     umma::bulk_g2s(smem + T::OFF_GEO, a.geo + kb * G_STRIDE, nb * G_STRIDE * 4u, barF);
-    umma::bulk_g2s(s_face, a.fcon + kb * 16, nb * 256u, barF);
+    umma::bulk_g2s(s_face, a.fcon + kb * 12, nb * 192u, barF);
   };
   if (tid == 0 && int(blockIdx.x) < tm.ntiles) {
     stage_rows(blockIdx.x);
@@ -345,13 +347,13 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
       const int64_t k = k0 + e;
       float contrib = 0.f;
       if (it < ne * NFF) {
-        const float4 *fr = s_face + (e * 4 + f) * 4;
-        const float4 r0 = fr[0], r1 = fr[1], r2 = fr[2], r3 = fr[3];
+        const float4 *fr = s_face + (e * 4 + f) * 3;
+        const float4 r0 = fr[0], r1 = fr[1], r2 = fr[2];
         const float n[3] = {r0.x, r0.y, r0.z};
-        const float zs = r0.w, Z2 = r1.y, Y2 = r1.w, ys = r2.x;
-        const int cny = __float_as_int(r2.w);
-        const int64_t k2 = __float_as_int(r3.x);
-        const bool wall = __float_as_int(r3.y) != 0;
+        const float zs = r0.w, Z2 = r1.x, Y2 = r1.y, ys = r1.z;
+        const int cny = __float_as_int(r1.w);
+        const int64_t k2 = __float_as_int(r2.z);
+        const bool wall = cny == kBoundaryConn;
         const int vm = s_fm[fm];
         const int fm2 = wall ? 0 : s_nf[cny * NFP + m] + (cny / 6 % 4) * NFP;
         const int vn = wall ? 0 : s_nb[cny * NFP + m];
@@ -377,7 +379,7 @@ __global__ void __launch_bounds__(AT<N>::NT, AT<N>::MINB)
         }
         float acc[6];
         const FaceNode fnode(n, gk, g2, Z2, Y2, zs, ys, a.alpha, acc);
-        if (grad) contrib = fnode.gradient(qm, qp, Z2, Y2, zs, ys, a.alpha, r2.y, r2.z);
+        if (grad) contrib = fnode.gradient(qm, qp, Z2, Y2, zs, ys, a.alpha, r2.x, r2.y);
         float2 *x = reinterpret_cast<float2 *>(s_x + fm * T::RSX + e * 6);
         x[0] = make_float2(acc[0], acc[1]);
         x[1] = make_float2(acc[2], acc[3]);
@@ -592,10 +594,9 @@ __global__ void k_adj_face_consts(int64_t K, const float *__restrict__ geo, cons
   const int64_t k2 = wall ? k : cn.x;
   const float Z2 = wall ? Zk : geo[k2 * G_STRIDE + G_Z], Y2 = wall ? Yk : geo[k2 * G_STRIDE + G_Y];
   const float ek = 1.f / geo[k * G_STRIDE + G_IEPS];
-  out[t * 4 + 0] = make_float4(nf.x, nf.y, nf.z, 1.f / (Zk + Z2));
-  out[t * 4 + 1] = make_float4(Zk, Z2, Yk, Y2);
-  out[t * 4 + 2] = make_float4(1.f / (Yk + Y2), -Zk / (2.f * ek), Yk / (2.f * ek), __int_as_float(cn.y));
-  out[t * 4 + 3] = make_float4(__int_as_float(int(k2)), __int_as_float(wall ? 1 : 0), 0.f, 0.f);
+  out[t * 3 + 0] = make_float4(nf.x, nf.y, nf.z, 1.f / (Zk + Z2));
+  out[t * 3 + 1] = make_float4(Z2, Y2, 1.f / (Yk + Y2), __int_as_float(cn.y));
+  out[t * 3 + 2] = make_float4(-Zk / (2.f * ek), Yk / (2.f * ek), __int_as_float(int(k2)), 0.f);
 }
 
 // Host: D^T and LIFT^T in the canonical K-major operand layout (FP16 hi, then
