@@ -29,7 +29,14 @@
 // 131,712 tets 203 -> 145; N=4 82,944 tets 298 -> 206; N=5 82,944 tets 479 ->
 // 395; N=6 24,576 tets 292 -> 227; N=7 24,576 tets 522 -> 422; N=8 24,576 tets
 // 859 -> 685; N=9 10,368 tets 668 -> 507; 162 tets at N=3 14.8 -> 6.6, 1,296
-// tets at N=5 21.1 -> 14.4.
+// tets at N=5 21.1 -> 14.6. A 36-element tile at N=5 takes 110k cycles, three
+// blocks sharing the SM: flux build 26k, products 44k, volume build 16k, update
+// 13k, face data 5k, barriers and operator copies 7k.
+//
+// The shape of two elements per thread sits at its limit of 168 registers and
+// spills a little in the update (bytes stored / loaded): 8-24 / 16-40, the store
+// form of the gradients' forward sweeps 104-152 / 112-276, the ensemble's tiles at
+// N = 4 and 7 40-60 / 60-72; the shapes of one element per thread spill nothing.
 #pragma once
 #include <atomic>
 #include <cmath>
@@ -327,7 +334,7 @@ __device__ __forceinline__ void simt_stage_tile(const StageArgs &a, int64_t k0, 
   // neither the rounded combinations nor the sums carry its rounding error
   // (right-hand side at N=5 against 64 bits: 1.5e-6 with it, 9.5e-7 with
   // differences from one node, 5.1e-7 now; 8.7e-7 with the combinations taken
-  // after the differentiation; N=3: 3.7e-7, 2.6e-7 now and 3.1e-7).
+  // after the differentiation; N=3: 3.7e-7, 2.5e-7 now and 3.1e-7).
 #pragma unroll 1
   for (int q0 = 0; q0 < NQ; q0 += QC) {
     __syncthreads(); // the previous product has read X and the operator rows

@@ -120,8 +120,12 @@ struct TC {
   // latencies; where a tile, the operators and the tensor memory columns of
   // several blocks fit, the other blocks' tiles fill the gaps, and half the
   // threads per block keep their registers. Two blocks at N = 4 would need
-  // 2 x 137 KB of shared memory. At N = 2 four blocks are faster on large meshes
-  // (80 us) but slower below 5,000 elements. Measured (FP16x3, us per stage, one
+  // 2 x 137 KB of shared memory, where an SM has 228, and 2 x 512 tensor memory
+  // columns, where it has 512 (a block uses 288; allocations are powers of two). At
+  // N = 2 four blocks are faster on large meshes (80 us) but slower below 5,000
+  // elements. The ensemble form keeps one block of 512 threads at every order: the
+  // occupancy query, and with it a cooperative launch, allows one block per SM of
+  // a kernel with tensor memory (so it was observed; no documentation says why). Measured (FP16x3, us per stage, one
   // block of 512 threads and now): N=1 162,000 tets 125 -> 55; N=2 131,712 tets
   // 134 -> 89; N=3 131,712 tets 161 -> 115 (two blocks of 512 threads: 133).
   static constexpr int BLOCKS = N == 1 ? 4 : N <= 3 ? 2 : 1;

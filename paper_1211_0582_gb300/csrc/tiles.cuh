@@ -45,7 +45,8 @@ TileMap<FULL> make_tiles(int64_t K, int grid) {
 // N=5 1,520 tets 9.73 -> 8.01; N=7 912 tets 15.3 -> 15.1, but 1,520 tets 16.3 ->
 // 17.3: 12 elements at N = 6, 7. A right-hand side has no stage after it: on its
 // own it takes the same time either way up to 12 elements and longer from there
-// (FP16x3 N=4 760 tets 11.0 and 11.1, 1,216 tets 11.1 -> 12.6).
+// (FP16x3 N=4 760 tets 11.0 and 11.1, 1,216 tets 11.1 -> 12.6; only a chain of
+// nothing but right-hand sides gains there, 6.71 -> 5.89).
 template <int FULL>
 int small_mesh_blocks(int64_t K, int cap, int most = FULL) {
   return cap >= 2 && K <= int64_t(most) * (cap / 2) ? cap / 2 : cap;
