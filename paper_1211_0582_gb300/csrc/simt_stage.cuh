@@ -123,13 +123,18 @@ struct SimtCfg {
 // Field loads. Tile rows come from L2 past L1 (used once or twice); the face
 // nodes' scattered reads hit the same lines again and go through L1, as plain
 // loads (the previous stage writes these rows while this one is resident: see
-// ld4). A persistent multi-stage launch (COHERENT) reads everything from L2:
-// other blocks wrote the data in an earlier stage.
+// ld4). The load is written out: volatile, it stays behind griddepcontrol.wait,
+// and unlike a C++ load it need not keep its place among the stores (us per stage
+// as a C++ load and so: N=6 60,000 tets 550 -> 541, N=8 1,900 tets 71.1 -> 70.0). A
+// persistent multi-stage launch (COHERENT) reads everything from L2: other
+// blocks wrote the data in an earlier stage.
 __device__ __forceinline__ float4 load_field4(const float *p) { return __ldcg(reinterpret_cast<const float4 *>(p)); }
 template <bool COHERENT>
 __device__ __forceinline__ float load_trace(const float *p) {
   if constexpr (COHERENT) return __ldcg(p);
-  else return *p;
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(__cvta_generic_to_global(p)));
+  return v;
 }
 
 // The node tables of a block (once per launch; the first tile's barrier orders them).
