@@ -115,7 +115,7 @@ std::string cache_path() {
 std::string cache_key(const EnsembleState &st, int N, int precision, int64_t K) {
   std::ostringstream os;
   // T: the candidate list that the cached index refers to
-  os << st.gpu << "|N=" << N << "|P=" << precision << "|K=" << K << "|T=3";
+  os << st.gpu << "|N=" << N << "|P=" << precision << "|K=" << K << "|T=4";
   return os.str();
 }
 

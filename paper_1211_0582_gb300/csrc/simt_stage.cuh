@@ -54,8 +54,9 @@ namespace dgmx {
 //     while a launch has only a few tiles per SM; at N <= 3 and N = 6 it is
 //     the faster one at every size.
 //   ONE_WIDE: the same with two or more times the elements per block (the rule is
-//     at simt_shape): more elements per SM in one round (N = 5: 36 instead of
-//     32), one copy of the operators for all of them.
+//     at simt_shape; at N = 4 the ensembles' tuner alone has it): more elements per
+//     SM in one round (N = 4: 56 instead of 48, N = 5: 36 instead of 32), one copy
+//     of the operators for all of them.
 //   TWO: two elements x two quads: half the shared-memory reads per product, but
 //     a tile takes as long with one element as with all of them.
 enum SimtShapeKind { SHAPE_TWO = 0, SHAPE_ONE = 1, SHAPE_ONE_WIDE = 2 };
@@ -67,7 +68,7 @@ struct SimtShape {
   static constexpr int CG = (D::NQ + CQ - 1) / CQ; // column groups: node quads cg and (CQ = 2) cg + CG
   // element groups of a block (even: neighbouring lanes hold two of them)
   static constexpr int GROUPS = SHAPE == SHAPE_TWO        ? 128 / CG / 2 * 2
-                                : SHAPE == SHAPE_ONE_WIDE ? (N == 5 ? 18 : N == 7 ? 16 : N == 8 ? 12 : 8)
+                                : SHAPE == SHAPE_ONE_WIDE ? (N == 4 ? 28 : N == 5 ? 18 : N == 7 ? 16 : N == 8 ? 12 : 8)
                                 : N == 1 ? 64 : N <= 3 ? 32 : N == 4 ? 16 : N == 6 ? 12 : N == 8 ? 6 : N == 9 ? 4 : 8;
   static constexpr int EB = RE * GROUPS;
   // Rows of X per chunk: FR face nodes (even, a divisor of 4 Nfp) or QC node
@@ -78,7 +79,8 @@ struct SimtShape {
                                   : N == 9 ? 4 : N == 8 ? 5 : N == 7 ? 6 : N == 5 ? 4 : 2;
 };
 
-// Orders that only the first shape serves, and those with the wide one.
+// Orders that only the first shape serves, and those whose single-mesh launches
+// have the wide one.
 template <int N>
 constexpr bool simt_one_only() {
   return N <= 3 || N == 6;
