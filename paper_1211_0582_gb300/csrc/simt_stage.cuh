@@ -52,11 +52,11 @@ namespace dgmx {
 //   ONE: one element x one quad and few, long chunks. A thread's chain of
 //     products and a tile's chain of barriers are short, which is what counts
 //     while a launch has only a few tiles per SM; at N <= 3 and N = 6 it is
-//     the faster one at every size.
+//     faster than TWO at every size.
 //   ONE_WIDE: the same with two or more times the elements per block (the rule is
 //     at simt_shape; at N = 4 the ensembles' tuner alone has it): more elements per
-//     SM in one round (N = 4: 56 instead of 48, N = 5: 36 instead of 32), one copy
-//     of the operators for all of them.
+//     SM in one round (N = 3: 100 instead of 96, N = 4: 56 instead of 48, N = 5: 36
+//     instead of 32), one copy of the operators for all of them.
 //   TWO: two elements x two quads: half the shared-memory reads per product, but
 //     a tile takes as long with one element as with all of them.
 enum SimtShapeKind { SHAPE_TWO = 0, SHAPE_ONE = 1, SHAPE_ONE_WIDE = 2 };
@@ -68,7 +68,7 @@ struct SimtShape {
   static constexpr int CG = (D::NQ + CQ - 1) / CQ; // column groups: node quads cg and (CQ = 2) cg + CG
   // element groups of a block (even: neighbouring lanes hold two of them)
   static constexpr int GROUPS = SHAPE == SHAPE_TWO        ? 128 / CG / 2 * 2
-                                : SHAPE == SHAPE_ONE_WIDE ? (N == 4 ? 28 : N == 5 ? 18 : N == 7 ? 16 : N == 8 ? 12 : 8)
+                                : SHAPE == SHAPE_ONE_WIDE ? (N == 3 ? 50 : N == 4 ? 28 : N == 5 ? 18 : N == 7 ? 16 : N == 8 ? 12 : 8)
                                 : N == 1 ? 64 : N <= 3 ? 32 : N == 4 ? 16 : N == 6 ? 12 : N == 8 ? 6 : N == 9 ? 4 : 8;
   static constexpr int EB = RE * GROUPS;
   // Rows of X per chunk: FR face nodes (even, a divisor of 4 Nfp) or QC node
@@ -79,15 +79,15 @@ struct SimtShape {
                                   : N == 9 ? 4 : N == 8 ? 5 : N == 7 ? 6 : N == 5 ? 4 : 2;
 };
 
-// Orders that only the first shape serves, and those whose single-mesh launches
-// have the wide one.
+// Orders without the two-element shape, and those whose single-mesh launches have
+// the wide one.
 template <int N>
 constexpr bool simt_one_only() {
   return N <= 3 || N == 6;
 }
 template <int N>
 constexpr bool simt_has_wide() {
-  return N == 5 || N >= 7;
+  return N == 3 || N == 5 || N >= 7;
 }
 
 template <int N, int SHAPE, int EB_ = SimtShape<N, SHAPE>::EB>
@@ -503,7 +503,8 @@ cudaError_t launch_simt_mode(const StageArgs &a, int dev, int sms, cudaStream_t 
 // tets 54.8 -> 43.6, 2,535 tets 111 -> 88; N=9 670 tets 72.5 -> 56.5, 2,590 tets 189 ->
 // 170). At N >= 7 not where few elements are left after whole rounds: the narrow
 // blocks do those beside other blocks' full tiles (N=8 1,875 tets 69.5, wide 79.2;
-// 1,995 tets 92.1, wide 79.6).
+// 1,995 tets 92.1, wide 79.6). At N = 3 where it takes a round less (15,000 tets 22.4
+// -> 17.6; 23,000 tets, two rounds either way, 27.5 and 28.1).
 template <int N>
 constexpr double simt_round_ratio() {
   return N == 4 ? 1.22 : N == 7 ? 1.24 : 1.35;
@@ -516,8 +517,13 @@ int simt_shape(int64_t K, int sms) {
   }
   if constexpr (simt_has_wide<N>()) {
     using One = SimtCfg<N, SHAPE_ONE>;
+    using Wide = SimtCfg<N, SHAPE_ONE_WIDE>;
+    if (N == 3) {
+      const int64_t one = int64_t(One::EB) * One::MINB * sms, wide = int64_t(Wide::EB) * Wide::MINB * sms;
+      return (K - 1) / wide < (K - 1) / one ? SHAPE_ONE_WIDE : SHAPE_ONE;
+    }
     const int64_t round = int64_t(One::EB) * (N == 5 ? One::MINB / 2 : 1) * sms;
-    const int64_t wide = int64_t(SimtShape<N, SHAPE_ONE_WIDE>::EB) * sms; // N >= 7: a round of the wide shape
+    const int64_t wide = int64_t(Wide::EB) * sms; // N >= 7: a round of the wide shape
     if (K > round) {
       if (N == 5) return (K - 1) / (int64_t(One::MINB) * sms) + 1 == 6 ? SHAPE_ONE : SHAPE_ONE_WIDE;
       const int64_t left = K % wide;
