@@ -135,7 +135,7 @@ template <bool COHERENT>
 __device__ __forceinline__ float load_trace(const float *p) {
   if constexpr (COHERENT) return __ldcg(p);
   float v;
-  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(__cvta_generic_to_global(p)));
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
   return v;
 }
 
