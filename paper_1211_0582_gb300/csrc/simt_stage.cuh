@@ -503,8 +503,10 @@ cudaError_t launch_simt_mode(const StageArgs &a, int dev, int sms, cudaStream_t 
 // tets 54.8 -> 43.6, 2,535 tets 111 -> 88; N=9 670 tets 72.5 -> 56.5, 2,590 tets 189 ->
 // 170). At N >= 7 not where few elements are left after whole rounds: the narrow
 // blocks do those beside other blocks' full tiles (N=8 1,875 tets 69.5, wide 79.2;
-// 1,995 tets 92.1, wide 79.6). At N = 3 where it takes a round less (15,000 tets 22.4
-// -> 17.6; 23,000 tets, two rounds either way, 27.5 and 28.1).
+// 1,995 tets 92.1, wide 79.6). At N = 3 where it takes one, two or three rounds
+// instead of one more (15,000 tets 22.4 -> 17.6, 45,000 tets 53.0 -> 48.5; with eight
+// instead of nine 117,000 tets 128 -> 129, and 23,000 tets, two either way, 27.5 ->
+// 28.1).
 template <int N>
 constexpr double simt_round_ratio() {
   return N == 4 ? 1.22 : N == 7 ? 1.24 : 1.35;
@@ -520,7 +522,7 @@ int simt_shape(int64_t K, int sms) {
     using Wide = SimtCfg<N, SHAPE_ONE_WIDE>;
     if (N == 3) {
       const int64_t one = int64_t(One::EB) * One::MINB * sms, wide = int64_t(Wide::EB) * Wide::MINB * sms;
-      return (K - 1) / wide < (K - 1) / one ? SHAPE_ONE_WIDE : SHAPE_ONE;
+      return (K - 1) / wide < (K - 1) / one && K <= 3 * wide ? SHAPE_ONE_WIDE : SHAPE_ONE;
     }
     const int64_t round = int64_t(One::EB) * (N == 5 ? One::MINB / 2 : 1) * sms;
     const int64_t wide = int64_t(Wide::EB) * sms; // N >= 7: a round of the wide shape
